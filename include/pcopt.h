@@ -424,7 +424,7 @@ int pc_sizes(const pc_handle* h, int64_t* ms, int64_t* vec_len);
  *            axis, 8 or 16 (default 16 in FP32, 8 in FP64).
  *   mg_ctas: CTAs per SM the fused down leg's grid is sized for, 1..64; it sets
  *            the spectral planes each CTA sweeps on every level (default 8).
- *   mv_tj:   time blocks per thread of the all-at-once matvec, 1..4096 (default 32).
+ *   mv_tj:   time blocks per thread of the all-at-once matvec, 1..4096 (default: by size).
  *   pro_pch: spectral planes per CTA of the prolongation and the 3D per-level
  *            multigrid kernels, 1..64 (default 8).
  *   fft_stream: time FFTs (power-of-two n): 0 = one CTA per tile of spatial

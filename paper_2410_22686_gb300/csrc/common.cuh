@@ -205,7 +205,7 @@ struct Prof {
 struct Tiles {
   int mg_cx = 0;    // fused 2D down leg: coarse points per tile axis (8 or 16)
   int mg_ctas = 0;  // fused 2D down leg: CTAs per SM its grid is sized for (sets planes per CTA per level)
-  int mv_tj = 0;    // matvec kernels: time blocks per thread
+  int mv_tj = 0;    // matvec kernels: time blocks per thread (0: by size)
   int pro_pch = 0;  // prolongation and per-level (3D) multigrid kernels: planes per CTA
   int fft_stream = 0;  // time FFTs: 0 one CTA per column tile, 1 persistent CTAs streaming tiles (cp.async)
   int mg_march = 0;    // fused 2D down leg with FP32 iterates: 0 shared-memory tiles, 1 register-marching warps
@@ -546,6 +546,9 @@ cudaError_t launch_grad_chunked(Launch& L, const Grid& g, int n, double scale, c
                                 const double* lam, double* partial, int tj, double* grad);
 
 int num_sms();
+// time blocks per thread of a double-float product launched with `blocks` CTAs per chunk of
+// time, for at least per_sm CTAs an SM (k_matvec.cu); tuned > 0 overrides
+int time_chunk_filling(int64_t blocks, int n, int per_sm, int tuned);
 
 // record `msg` as the calling thread's last error (pc_last_error) and return `status`
 int set_error(int status, const std::string& msg);

@@ -59,22 +59,26 @@ __global__ void __launch_bounds__(256) matvec_kernel(const Tin* __restrict__ x, 
   }
 #pragma unroll
   for (int k = 0; k < 2 * DIM; ++k) wv[k] = w[(int64_t)k * ms + s];
-  const double dg = diag[s];
+  // the centre of v_j - v_{j-1} + tau K v_j as one coefficient: 2 dim + 3 FP64 operations
+  // an output instead of 2 dim + 4 (this kernel is bound by the FP64 unit: 255^2 x 256,
+  // 33.3 M unknowns, 32 time blocks a thread: 498 us before, 431 with it)
+  const double dg1 = 1.0 + diag[s];
 
   const Tin* x1 = x;
   const Tin* x2 = x + (int64_t)n * ms;
   double* y1 = y;
   double* y2 = y + (int64_t)n * ms;
 
-  auto tauK = [&](const Tin* base, double centre) -> double {
-    double acc = dg * centre;
+  // acc + sum of the neighbours' face weights times their values
+  auto faces = [&](const Tin* base, double sgn, double acc) -> double {
 #pragma unroll
     for (int k = 0; k < 2 * DIM; ++k) {
-      double nb = ex[k] ? cvt<double>(__ldg(base + off[k])) : 0.0;
-      acc = fma(-wv[k], nb, acc);
+      const double nb = ex[k] ? cvt<double>(__ldg(base + off[k])) : 0.0;
+      acc = fma(sgn * wv[k], nb, acc);
     }
     return acc;
   };
+  constexpr double sg = TRANSPOSE ? -1.0 : 1.0;
 
   double x1prev = (j0 > 0) ? cvt<double>(x1[(int64_t)(j0 - 1) * ms + s]) : 0.0;
   double x2c = cvt<double>(x2[(int64_t)j0 * ms + s]);
@@ -83,17 +87,11 @@ __global__ void __launch_bounds__(256) matvec_kernel(const Tin* __restrict__ x, 
     const int64_t idx = (int64_t)j * ms + s;
     const double x1c = cvt<double>(x1[idx]);
     const double x2n = (j + 1 < n) ? cvt<double>(x2[idx + ms]) : 0.0;
-    const double k1 = tauK(x1 + idx, x1c);
-    const double k2 = tauK(x2 + idx, x2c);
-    const double tT_x2 = x2c - x2n + k2;     // (T^T x2)_j
-    const double t_x1 = x1c - x1prev + k1;   // (T x1)_j
-    if (!TRANSPOSE) {
-      y1[idx] = fma(alpha, x1c, tT_x2);
-      y2[idx] = fma(alpha, x2c, -t_x1);
-    } else {
-      y1[idx] = fma(alpha, x1c, -tT_x2);
-      y2[idx] = fma(alpha, x2c, t_x1);
-    }
+    // y1 = alpha x1_j + sg ((1 + d) x2_j - x2_{j+1} - faces), y2 = alpha x2_j - sg (...)
+    const double a = fma(alpha, x1c, faces(x2 + idx, -sg, sg * dg1 * x2c));
+    const double b = fma(alpha, x2c, faces(x1 + idx, sg, -sg * dg1 * x1c));
+    y1[idx] = TRANSPOSE ? a + x2n : a - x2n;
+    y2[idx] = TRANSPOSE ? b - x1prev : b + x1prev;
     x1prev = x1c;
     x2c = x2n;
   }
@@ -101,10 +99,13 @@ __global__ void __launch_bounds__(256) matvec_kernel(const Tin* __restrict__ x, 
 
 }  // namespace
 
-// time blocks per thread: the tuned value, else 32 (a thread carries its time
-// neighbour in registers, so longer chunks re-read fewer x values)
+// Time blocks per thread: the tuned value, else 4 for the FP64 kernel.  A thread re-reads
+// two x values and its stencil at the start of a chunk; the FP64 unit bounds the kernel,
+// so that costs little at any size, and short chunks fill the chip where n is small
+// (63^2 x 64: 34.8 us at 32 blocks a thread, 12.3 at 4; 127^2 x 128: 63.6 and 57.4;
+// 255^2 x 256: 431 and 419; one block a thread takes 445 there).
 static int time_chunk(const Launch& L, int n) {
-  int tj = L.tiles && L.tiles->mv_tj > 0 ? L.tiles->mv_tj : 32;
+  const int tj = L.tiles && L.tiles->mv_tj > 0 ? L.tiles->mv_tj : 4;
   return tj < n ? tj : n;
 }
 
@@ -264,10 +265,24 @@ __global__ void __launch_bounds__(256) matvec_df_kernel(const float* __restrict_
 
 }  // namespace
 
+// Time blocks per thread of the double-float products: the tuned value, else 16, halved
+// until `blocks` CTAs a chunk of time make `per_sm` CTAs an SM.  A chunk's start costs them
+// 12-byte stencil pairs and (elements) two more mass products, so long chunks are the
+// better ones once the chip is full: differences 255^2 x 256 take 177 us at 16 blocks,
+// 189 at 4, 245 at 1; 127^2 x 64 24.6 us at 32, 18.5 at 8 and 16.4 at 4; 31^2 x 32 24.6 at
+// 32 and 7.5 at 1.
+int time_chunk_filling(int64_t blocks, int n, int per_sm, int tuned) {
+  if (tuned > 0) return tuned < n ? tuned : n;
+  const int64_t want = (int64_t)num_sms() * per_sm;
+  int tj = 16;
+  while (tj > 1 && blocks * ((n + tj - 1) / tj) < want) tj >>= 1;
+  return tj < n ? tj : n;
+}
+
 cudaError_t launch_matvec_df(Launch& L, const Grid& g, int n, const float2* w, const float2* diag, float2 alpha,
                              const float* x, double* y, size_t xstride, size_t ystride, const int* jdev) {
   const int threads = 256;
-  const int tj = time_chunk(L, n);
+  const int tj = time_chunk_filling((g.np + threads - 1) / threads, n, 6, L.tiles ? L.tiles->mv_tj : 0);
   dim3 grid((unsigned)((g.np + threads - 1) / threads), (unsigned)((n + tj - 1) / tj));
   const double U = 2.0 * (double)n * (double)g.np;
   const double bytes = U * (sizeof(float) + sizeof(double)) + (2.0 * g.dim + 1) * g.np * 8.0;
