@@ -194,6 +194,8 @@ struct pc_handle {
   double2* sig1_64 = nullptr;  // the shift 1 (end-point solves)
   float2* sig1_32 = nullptr;
   float2* sig32 = nullptr;
+  void* cz_tab = nullptr;  // chirp-z table of the handle's precision (n not a power of two)
+  int cz_logM = 0;
   // ideal RBD preconditioner (Eq. matrix_P): the real shift 1 + alpha of both planes
   int precond_kind = PC_PRECOND_EPS_CIRCULANT;
   int arnoldi = PC_ARNOLDI_AUTO;  // pc_arnoldi: basis storage and product precision of flexible GMRES
@@ -492,6 +494,60 @@ static int upload_c(pc_handle* h, void** dst, const std::vector<double>& re, con
   return PC_OK;
 }
 
+// in-place DFT of 2^b values (radix 2, kernel exp(-2 pi i jk / 2^b)), cs/sn the circle's
+// cosines and sines
+static void host_fft(std::vector<double>& re, std::vector<double>& im, int b, const std::vector<double>& cs,
+                     const std::vector<double>& sn) {
+  const int M = 1 << b;
+  for (int i = 1, j = 0; i < M; ++i) {
+    int bit = M >> 1;
+    for (; j & bit; bit >>= 1) j ^= bit;
+    j ^= bit;
+    if (i < j) {
+      std::swap(re[i], re[j]);
+      std::swap(im[i], im[j]);
+    }
+  }
+  for (int half = 1; half < M; half <<= 1)
+    for (int g = 0; g < M; g += 2 * half)
+      for (int p = 0; p < half; ++p) {
+        const double c = cs[(size_t)p * (M / (2 * half))], s = -sn[(size_t)p * (M / (2 * half))];
+        const int i = g + p, k = i + half;
+        const double br = c * re[k] - s * im[k], bi = c * im[k] + s * re[k];
+        re[k] = re[i] - br;
+        im[k] = im[i] - bi;
+        re[i] += br;
+        im[i] += bi;
+      }
+}
+
+// the table of ChirpZ for length n, M = 2^b
+static void chirp_table(int n, int b, std::vector<double>& re, std::vector<double>& im) {
+  const int M = 1 << b;
+  std::vector<double> cs(M), sn(M), hr(M, 0.0), hi(M, 0.0);
+  for (int q = 0; q < M; ++q) {
+    cs[q] = std::cos(2.0 * M_PI * q / M);
+    sn[q] = std::sin(2.0 * M_PI * q / M);
+  }
+  re.assign((size_t)n + 2 * M, 0.0);
+  im.assign((size_t)n + 2 * M, 0.0);
+  for (int j = 0; j < n; ++j) {
+    const double th = M_PI * (double)((int64_t)j * j % (2 * n)) / n;  // j^2 mod 2n: the angle's exact period
+    re[j] = std::cos(th);
+    im[j] = -std::sin(th);
+    hr[j] = hr[(M - j) % M] = re[j];
+    hi[j] = hi[(M - j) % M] = -im[j];
+  }
+  host_fft(hr, hi, b, cs, sn);
+  for (int k = 0; k < M; ++k) {
+    const size_t at = (size_t)n + chirp_position(b, k);
+    re[at] = hr[k] / M;
+    im[at] = hi[k] / M;
+    re[(size_t)n + M + k] = cs[k];
+    im[(size_t)n + M + k] = -sn[k];
+  }
+}
+
 // bytes of the Krylov basis V (cap + 1 vectors of the tiled layout, 8 bytes per
 // unknown) and of the preconditioned vectors Z (cap vectors, FP32 or FP64), each
 // part rounded up to 256 bytes; Z follows V
@@ -737,6 +793,12 @@ static int setup_impl(const pc_params* p, const double* a_nodes, void* krylov, s
     const std::vector<double> shiftP(2, 1.0 + h->alpha), zero2(2, 0.0);
     if ((rc = upload_c(h, (void**)&h->sigP64, shiftP, zero2, false, st))) goto fail_out;
     if ((rc = upload_c(h, (void**)&h->sigP32, shiftP, zero2, true, st))) goto fail_out;
+  }
+  if (chirp_log2(h->n)) {
+    h->cz_logM = chirp_log2(h->n);
+    std::vector<double> re, im;
+    chirp_table(h->n, h->cz_logM, re, im);
+    if ((rc = upload_c(h, &h->cz_tab, re, im, h->fp32, st))) goto fail_out;
   }
   // ---- FST tables (constant a)
   if (spatial == PC_SPATIAL_FST) {
@@ -1235,12 +1297,19 @@ static cudaError_t precond_t(pc_handle* h, Launch& L, const Tin* v, Tout* w, siz
     if (stride != 0 || jdev != nullptr) return cudaErrorNotSupported;  // graph solves reject it first
     return precond_ideal_t<Tc, TU, Tout, Tin>(h, L, v, w);
   }
-  cudaError_t e = launch_tfft_forward<Tc>(L, h->ms, h->n, v, Tables<Tc>::dpow(h), Tables<Tc>::dinv(h),
-                                          Tables<Tc>::tw(h), (C*)h->lv[0].r,
-                                          index_input ? (in_stride ? in_stride : stride) : 0,
-                                          index_input ? jdev : nullptr);
+  // n not a power of two: the chirp-z transforms (host-driven solves only, so no index)
+  const ChirpZ<Tc> cz{(const C*)h->cz_tab, h->cz_logM};
+  if (cz.logM && jdev) return cudaErrorNotSupported;
+  cudaError_t e = cz.logM ? launch_tchirp_forward<Tc, Tin>(L, h->ms, h->n, v, Tables<Tc>::dpow(h), cz, (C*)h->lv[0].r)
+                          : launch_tfft_forward<Tc>(L, h->ms, h->n, v, Tables<Tc>::dpow(h), Tables<Tc>::dinv(h),
+                                                    Tables<Tc>::tw(h), (C*)h->lv[0].r,
+                                                    index_input ? (in_stride ? in_stride : stride) : 0,
+                                                    index_input ? jdev : nullptr);
   if (e != cudaSuccess) return e;
   if ((e = spatial_solve<Tc, TU>(h, L)) != cudaSuccess) return e;
+  if (cz.logM)
+    return launch_tchirp_inverse<Tc, TU, Tout>(L, h->ms, h->n, (const TU*)h->lv[0].u, Tables<Tc>::dinv(h), cz, w,
+                                               fine_correction<TU>(h));
   return launch_tfft_inverse<Tc, TU, Tout>(L, h->ms, h->n, (const TU*)h->lv[0].u, Tables<Tc>::dpow(h),
                                            Tables<Tc>::dinv(h), Tables<Tc>::tw(h), w, stride, jdev,
                                            fine_correction<TU>(h));

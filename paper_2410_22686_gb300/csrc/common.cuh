@@ -353,6 +353,28 @@ cudaError_t launch_tfft_inverse(Launch& L, int64_t ms, int n, const TU* spec, co
                                 const typename Cx<Tc>::t* tw, Tout* w, size_t wstride = 0,
                                 const int* jdev = nullptr, FineCorrection<TU> fc = FineCorrection<TU>());
 
+// Time transforms of lengths that are not powers of two by the chirp-z method
+// (k_tchirp.cu), n >= kChirpMinN (shorter ones take the direct sum of k_tfft.cu).  One
+// table: chirp c_j = exp(-pi i j^2 / n), j < n; filter = DFT_M(conj c) / M at
+// chirp_position; roots exp(-2 pi i q / M), q < M.  logM = 0: no table.
+constexpr int kChirpMinN = 24;
+template <typename T>
+struct ChirpZ {
+  const typename Cx<T>::t* tab = nullptr;
+  int logM = 0;
+  __device__ __forceinline__ const typename Cx<T>::t* chirp() const { return tab; }
+  __device__ __forceinline__ const typename Cx<T>::t* filter(int n) const { return tab + n; }
+  __device__ __forceinline__ const typename Cx<T>::t* roots(int n) const { return tab + n + (1 << logM); }
+};
+int chirp_log2(int n);                   // log2 M for length n, 0 where the method is not used
+int chirp_position(int logM, int k);     // where frequency k lies after the forward passes
+template <typename Tc, typename Tin>
+cudaError_t launch_tchirp_forward(Launch& L, int64_t ms, int n, const Tin* v, const Tc* dpow, ChirpZ<Tc> cz,
+                                  typename Cx<Tc>::t* spec);
+template <typename Tc, typename TU, typename Tout>
+cudaError_t launch_tchirp_inverse(Launch& L, int64_t ms, int n, const TU* spec, const Tc* dinv, ChirpZ<Tc> cz, Tout* w,
+                                  FineCorrection<TU> fc);
+
 // FST: one DST-I along `axis` of every plane (out = S in), and the spectral divide
 // buf *= rmass / (sigma + lamK) (rmass == nullptr: 1)
 template <typename Tc>

@@ -48,6 +48,77 @@ __device__ __forceinline__ void reg_fft(C (&x)[R], const C* __restrict__ tw, int
   }
 }
 
+// cos(2 pi q / 32) for q = 0..8
+template <typename T>
+__device__ __forceinline__ constexpr T cos32(int q) {
+  switch (q) {
+    case 0: return T(1);
+    case 1: return T(0.98078528040323044912618223613424);
+    case 2: return T(0.92387953251128675612818318939679);
+    case 3: return T(0.83146961230254523707878837761791);
+    case 4: return T(0.70710678118654752440084436210485);
+    case 5: return T(0.55557023301960222474283081394853);
+    case 6: return T(0.38268343236508977172845998403040);
+    case 7: return T(0.19509032201612826784828486847702);
+    default: return T(0);
+  }
+}
+
+// In-place R-point DFT of registers (R <= 32), the twiddles compile-time constants.  A
+// butterfly with a twiddle takes six fused multiply-adds (a + w b in four, and a - w b as
+// 2 a - (a + w b)) where a product and two sums take eight; quarter turns cost the sums
+// alone.  16 points: 148 operations instead of 196.  HALF_IN: inputs R/2.. are zero;
+// HALF_OUT: only outputs 0..R/2-1 are wanted.
+template <int R, bool INV, bool HALF_IN = false, bool HALF_OUT = false, typename C>
+__device__ __forceinline__ void dft_regs(C (&x)[R]) {
+  typedef decltype(C().x) T;
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const int j = brev_ct<R>(i);
+    if (j > i) {
+      const C t = x[i];
+      x[i] = x[j];
+      x[j] = t;
+    }
+  }
+#pragma unroll
+  for (int half = 1; half < R; half <<= 1) {
+    const bool last = HALF_OUT && 2 * half == R;
+#pragma unroll
+    for (int g = 0; g < R; g += 2 * half) {
+#pragma unroll
+      for (int p = 0; p < half; ++p) {
+        const C a = x[g + p], b = x[g + p + half];
+        if (HALF_IN && half == 1) {
+          x[g + 1] = a;
+        } else if (p == 0) {
+          x[g + p] = a + b;
+          if (!last) x[g + p + half] = a - b;
+        } else if (2 * p == half) {  // w = -i (forward), i (inverse)
+          C t;
+          t.x = INV ? -b.y : b.y;
+          t.y = INV ? b.x : -b.x;
+          x[g + p] = a + t;
+          if (!last) x[g + p + half] = a - t;
+        } else {
+          const int q = p * (16 / half);  // w = exp(-+ 2 pi i q / 32), 0 < q < 16
+          const T wr = q <= 8 ? cos32<T>(q) : -cos32<T>(16 - q);
+          const T ws = q <= 8 ? cos32<T>(8 - q) : cos32<T>(q - 8);
+          const T wi = INV ? ws : -ws;
+          C t;
+          t.x = fma(-wi, b.y, fma(wr, b.x, a.x));
+          t.y = fma(wi, b.x, fma(wr, b.y, a.y));
+          x[g + p] = t;
+          if (!last) {
+            x[g + p + half].x = fma(T(2), a.x, -t.x);
+            x[g + p + half].y = fma(T(2), a.y, -t.y);
+          }
+        }
+      }
+    }
+  }
+}
+
 // cp.async (sm_80+ asynchronous global -> shared copy of B = 4, 8 or 16 bytes,
 // bypassing registers); `ok == false` zero-fills the destination without reading
 // global memory
