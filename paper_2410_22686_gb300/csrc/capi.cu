@@ -740,7 +740,9 @@ static int setup_impl(const pc_params* p, const double* a_nodes, void* krylov, s
     // per plane made the ideal preconditioner's two-plane steps slower: 29.6 -> 34.8
     // ms per apply at 255^2 x 256.)
     h->tail2 = dim == 2 && h->fp32 && !h->bf16s && !h->fevar;
-    const int mthr = h->tail2 ? kMgTailMaxM : (dim == 2 ? 31 : 15);
+    // Element multigrid in 2D: from 63^2 in FP32 (74 KB of shared memory), 31^2 in FP64.
+    const bool tail63 = h->tail2 || (h->fevar && dim == 2 && h->fp32);
+    const int mthr = tail63 ? kMgTailMaxM : (dim == 2 ? 31 : 15);
     int l0 = (int)h->lv.size() - 1;
     while (l0 > 0 && h->lv[l0 - 1].m <= mthr) --l0;
     if ((int)h->lv.size() - l0 > kMaxCoarseLevels) l0 = (int)h->lv.size() - kMaxCoarseLevels;
@@ -1074,20 +1076,27 @@ const double* lve<double>(const LevelBuf& L) { return L.e64; }
 template <>
 const float* lve<float>(const LevelBuf& L) { return L.e32; }
 
-// element multigrid (k_fevar.cu in 2D, k_fevar3.cu in 3D): on every level a
-// colour-ordered Gauss-Seidel sweep from zero, residual and restriction by P^T; the
-// one-point level is solved by its sweep; then the (bi/tri)linear corrections from the
-// coarsest level up
+// element multigrid: a colour-ordered Gauss-Seidel sweep from zero, residual and restriction
+// by P^T on the way down, the one-point level solved by its sweep, the (bi/tri)linear
+// corrections on the way up.  2D (k_femg.cu): a launch per fine level and one for the levels
+// from coarse_l0 down and back; the finest correction is left to the inverse time transform
+// unless `complete`.  3D (k_fevar3.cu) and 2D levels too wide for a strip: per-level kernels.
 template <typename Tc>
-static cudaError_t fevar_spatial(pc_handle* h, Launch& L, int P, const typename Cx<Tc>::t* sig) {
+static cudaError_t fevar_spatial(pc_handle* h, Launch& L, int P, const typename Cx<Tc>::t* sig, bool complete) {
   typedef typename Cx<Tc>::t C;
   const int nl = (int)h->lv.size();
+  const int l0 = h->dim == 2 ? h->coarse_l0 : nl;  // first level of the fused lower cycle
   const Tc tau = (Tc)h->tau;
   cudaError_t e;
-  for (int l = 0; l < nl; ++l) {
+  for (int l = 0; l < l0; ++l) {
     const LevelBuf& B = h->lv[l];
     const Tc hl = Tc(1) / Tc(B.m + 1);
     const Tc* E = lve<Tc>(B);
+    if (h->dim == 2 && fe_down_rows<Tc>(B.m, P) > 0) {
+      e = launch_fe_down<Tc>(L, B.m, P, hl * hl, tau, E, sig, (const C*)B.r, (C*)B.u, (C*)h->lv[l + 1].r);
+      if (e != cudaSuccess) return e;
+      continue;
+    }
     e = h->dim == 3 ? launch_fevar3_smooth<Tc>(L, B.m, P, hl, tau, E, sig, (const C*)B.r, (C*)B.u)
                     : launch_fevar_smooth<Tc>(L, B.m, P, hl * hl, tau, E, sig, (const C*)B.r, (C*)B.u);
     if (e != cudaSuccess) return e;
@@ -1098,7 +1107,18 @@ static cudaError_t fevar_spatial(pc_handle* h, Launch& L, int P, const typename 
                                                       (const C*)B.u, (C*)B.res, (C*)h->lv[l + 1].r);
     if (e != cudaSuccess) return e;
   }
-  for (int l = nl - 2; l >= 0; --l)
+  if (l0 < nl) {
+    FeLevels<Tc> lv{};
+    lv.count = nl - l0;
+    for (int l = l0; l < nl; ++l) {
+      lv.m[l - l0] = h->lv[l].m;
+      lv.E[l - l0] = lve<Tc>(h->lv[l]);
+    }
+    e = launch_fe_tail<Tc>(L, P, lv, tau, sig, (const C*)h->lv[l0].r, (C*)h->lv[l0].u);
+    if (e != cudaSuccess) return e;
+  }
+  const int up = std::min(l0, nl - 1) - 1, last = h->dim == 2 && !complete ? 1 : 0;
+  for (int l = up; l >= last; --l)
     if ((e = launch_mg_prolong<Tc, C>(L, grid_of(h, l), P, (const C*)h->lv[l + 1].u, (C*)h->lv[l].u)) != cudaSuccess)
       return e;
   return cudaSuccess;
@@ -1189,7 +1209,7 @@ static cudaError_t spatial_solve(pc_handle* h, Launch& L, int nplanes = 0,
     }
   }
   if (h->fevar) {
-    if constexpr (std::is_same<TU, C>::value) return fevar_spatial<Tc>(h, L, P, sig);
+    if constexpr (std::is_same<TU, C>::value) return fevar_spatial<Tc>(h, L, P, sig, complete);
     return cudaErrorNotSupported;
   }
   // multigrid V(1,0): per-level kernels on the fine levels, one fused kernel for the rest
@@ -1258,7 +1278,7 @@ static cudaError_t spatial_solve(pc_handle* h, Launch& L, int nplanes = 0,
 template <typename TU>
 static FineCorrection<TU> fine_correction(const pc_handle* h) {
   FineCorrection<TU> fc;
-  if (h->spatial == PC_SPATIAL_FST || h->lex || h->fevar || h->coarse_l0 < 1 || h->dim != 2) return fc;
+  if (h->spatial == PC_SPATIAL_FST || h->lex || h->coarse_l0 < 1 || h->dim != 2) return fc;
   const Grid g0 = grid_of(h, 0), g1 = grid_of(h, 1);
   fc.ec = (const TU*)h->lv[1].u;
   fc.dim = h->dim;

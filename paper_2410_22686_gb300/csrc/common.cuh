@@ -432,6 +432,23 @@ struct CoarseLevels {
   const T* w[kMaxCoarseLevels];
   const T* diag[kMaxCoarseLevels];
 };
+// Element multigrid in 2D (k_femg.cu): one level's sweep, residual and restriction by P^T in
+// one launch (fe_down_rows: coarse rows per strip, 0 where a strip does not fit), and the
+// levels from lv.m[0] <= 63 down and back up in another
+template <typename T>
+struct FeLevels {
+  int count;
+  int m[kMaxCoarseLevels];
+  const T* E[kMaxCoarseLevels];
+};
+template <typename Tc>
+int fe_down_rows(int m, int planes);
+template <typename Tc>
+cudaError_t launch_fe_down(Launch& L, int m, int planes, Tc h2, Tc tau, const Tc* E, const typename Cx<Tc>::t* sigma,
+                           const typename Cx<Tc>::t* r, typename Cx<Tc>::t* u, typename Cx<Tc>::t* rc);
+template <typename Tc>
+cudaError_t launch_fe_tail(Launch& L, int planes, const FeLevels<Tc>& lv, Tc tau, const typename Cx<Tc>::t* sigma,
+                           const typename Cx<Tc>::t* r, typename Cx<Tc>::t* u);
 // 2D FP32 iterates: the lower part of the cycle from the first level with
 // m <= kMgTailMaxM, one array per level updated in place (k_mgtail.cu)
 constexpr int kMgTailMaxM = 63;
