@@ -704,8 +704,11 @@ static int setup_impl(const pc_params* p, const double* a_nodes, void* krylov, s
       if ((rc = dev_alloc(h, &L.r, (size_t)h->planes * L.np * cb))) goto fail_out;
       if ((rc = dev_alloc(h, &L.u, (size_t)h->planes * L.np * ub))) goto fail_out;
       // per-level residual planes: the 3D path and the natural-order smoother write them
-      // (the 2D red-black down leg fuses the residual away)
-      if ((dim == 3 || h->lex || h->fevar) && l + 1 < mlev.size() &&
+      // (the 2D red-black down leg and the element levels' strips fuse the residual away)
+      const bool strips = h->fevar && (dim == 2 ? (h->fp32 ? fe_down_rows<float>(L.m, h->planes)
+                                                            : fe_down_rows<double>(L.m, h->planes)) > 0
+                                                : (h->fp32 ? fe3_down_fits<float>(L.m) : fe3_down_fits<double>(L.m)));
+      if ((dim == 3 || h->lex || h->fevar) && !strips && l + 1 < mlev.size() &&
           (rc = dev_alloc(h, &L.res, (size_t)h->planes * L.np * cb)))
         goto fail_out;
       h->lv.push_back(L);
@@ -1078,50 +1081,47 @@ const float* lve<float>(const LevelBuf& L) { return L.e32; }
 
 // element multigrid: a colour-ordered Gauss-Seidel sweep from zero, residual and restriction
 // by P^T on the way down, the one-point level solved by its sweep, the (bi/tri)linear
-// corrections on the way up.  2D (k_femg.cu): a launch per fine level and one for the levels
-// from coarse_l0 down and back; the finest correction is left to the inverse time transform
-// unless `complete`.  3D (k_fevar3.cu) and 2D levels too wide for a strip: per-level kernels.
+// corrections on the way up (k_femg.cu in 2D, k_femg3.cu in 3D): fused launches for each fine
+// level and one for the levels from coarse_l0 down and back.  In 2D the finest correction is
+// left to the inverse time transform unless `complete`.  Levels too wide for a strip of rows
+// in shared memory take the per-level kernels of k_fevar.cu and k_fevar3.cu.
 template <typename Tc>
 static cudaError_t fevar_spatial(pc_handle* h, Launch& L, int P, const typename Cx<Tc>::t* sig, bool complete) {
   typedef typename Cx<Tc>::t C;
-  const int nl = (int)h->lv.size();
-  const int l0 = h->dim == 2 ? h->coarse_l0 : nl;  // first level of the fused lower cycle
+  const int nl = (int)h->lv.size(), l0 = h->coarse_l0;
   const Tc tau = (Tc)h->tau;
   cudaError_t e;
   for (int l = 0; l < l0; ++l) {
     const LevelBuf& B = h->lv[l];
     const Tc hl = Tc(1) / Tc(B.m + 1);
     const Tc* E = lve<Tc>(B);
-    if (h->dim == 2 && fe_down_rows<Tc>(B.m, P) > 0) {
-      e = launch_fe_down<Tc>(L, B.m, P, hl * hl, tau, E, sig, (const C*)B.r, (C*)B.u, (C*)h->lv[l + 1].r);
-      if (e != cudaSuccess) return e;
-      continue;
+    const C* r = (const C*)B.r;
+    C *u = (C*)B.u, *res = (C*)B.res, *rc = (C*)h->lv[l + 1].r;
+    if (h->dim == 2) {
+      if (fe_down_rows<Tc>(B.m, P) > 0)
+        e = launch_fe_down<Tc>(L, B.m, P, hl * hl, tau, E, sig, r, u, rc);
+      else if ((e = launch_fevar_smooth<Tc>(L, B.m, P, hl * hl, tau, E, sig, r, u)) == cudaSuccess)
+        e = launch_fevar_resid_restrict<Tc>(L, B.m, P, hl * hl, tau, E, sig, r, u, res, rc);
+    } else {
+      if (fe3_down_fits<Tc>(B.m))
+        e = launch_fe3_down<Tc>(L, B.m, P, hl, tau, E, sig, r, u, rc);
+      else if ((e = launch_fevar3_smooth<Tc>(L, B.m, P, hl, tau, E, sig, r, u)) == cudaSuccess)
+        e = launch_fevar3_resid_restrict<Tc>(L, B.m, P, hl, tau, E, sig, r, u, res, rc);
     }
-    e = h->dim == 3 ? launch_fevar3_smooth<Tc>(L, B.m, P, hl, tau, E, sig, (const C*)B.r, (C*)B.u)
-                    : launch_fevar_smooth<Tc>(L, B.m, P, hl * hl, tau, E, sig, (const C*)B.r, (C*)B.u);
-    if (e != cudaSuccess) return e;
-    if (l + 1 == nl) break;
-    e = h->dim == 3 ? launch_fevar3_resid_restrict<Tc>(L, B.m, P, hl, tau, E, sig, (const C*)B.r, (const C*)B.u,
-                                                       (C*)B.res, (C*)h->lv[l + 1].r)
-                    : launch_fevar_resid_restrict<Tc>(L, B.m, P, hl * hl, tau, E, sig, (const C*)B.r,
-                                                      (const C*)B.u, (C*)B.res, (C*)h->lv[l + 1].r);
     if (e != cudaSuccess) return e;
   }
-  if (l0 < nl) {
-    FeLevels<Tc> lv{};
-    lv.count = nl - l0;
-    for (int l = l0; l < nl; ++l) {
-      lv.m[l - l0] = h->lv[l].m;
-      lv.E[l - l0] = lve<Tc>(h->lv[l]);
-    }
-    e = launch_fe_tail<Tc>(L, P, lv, tau, sig, (const C*)h->lv[l0].r, (C*)h->lv[l0].u);
-    if (e != cudaSuccess) return e;
+  FeLevels<Tc> lv{};
+  lv.count = nl - l0;
+  for (int l = l0; l < nl; ++l) {
+    lv.m[l - l0] = h->lv[l].m;
+    lv.E[l - l0] = lve<Tc>(h->lv[l]);
   }
-  const int up = std::min(l0, nl - 1) - 1, last = h->dim == 2 && !complete ? 1 : 0;
-  for (int l = up; l >= last; --l)
-    if ((e = launch_mg_prolong<Tc, C>(L, grid_of(h, l), P, (const C*)h->lv[l + 1].u, (C*)h->lv[l].u)) != cudaSuccess)
-      return e;
-  return cudaSuccess;
+  const C* r0 = (const C*)h->lv[l0].r;
+  C* u0 = (C*)h->lv[l0].u;
+  e = h->dim == 2 ? launch_fe_tail<Tc>(L, P, lv, tau, sig, r0, u0) : launch_fe3_tail<Tc>(L, P, lv, tau, sig, r0, u0);
+  for (int l = l0 - 1; e == cudaSuccess && l >= (h->dim == 2 && !complete ? 1 : 0); --l)
+    e = launch_mg_prolong<Tc, C>(L, grid_of(h, l), P, (const C*)h->lv[l + 1].u, (C*)h->lv[l].u);
+  return e;
 }
 
 template <typename Tc>

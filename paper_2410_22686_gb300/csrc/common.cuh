@@ -449,6 +449,15 @@ cudaError_t launch_fe_down(Launch& L, int m, int planes, Tc h2, Tc tau, const Tc
 template <typename Tc>
 cudaError_t launch_fe_tail(Launch& L, int planes, const FeLevels<Tc>& lv, Tc tau, const typename Cx<Tc>::t* sigma,
                            const typename Cx<Tc>::t* r, typename Cx<Tc>::t* u);
+// ... and in 3D (k_femg3.cu): even layers, odd layers, residual + restriction; lv.m[0] <= 15
+template <typename Tc>
+bool fe3_down_fits(int m);
+template <typename Tc>
+cudaError_t launch_fe3_down(Launch& L, int m, int planes, Tc h, Tc tau, const Tc* E, const typename Cx<Tc>::t* sigma,
+                            const typename Cx<Tc>::t* r, typename Cx<Tc>::t* u, typename Cx<Tc>::t* rc);
+template <typename Tc>
+cudaError_t launch_fe3_tail(Launch& L, int planes, const FeLevels<Tc>& lv, Tc tau, const typename Cx<Tc>::t* sigma,
+                            const typename Cx<Tc>::t* r, typename Cx<Tc>::t* u);
 // 2D FP32 iterates: the lower part of the cycle from the first level with
 // m <= kMgTailMaxM, one array per level updated in place (k_mgtail.cu)
 constexpr int kMgTailMaxM = 63;

@@ -1,8 +1,9 @@
 // Multigrid V(1,0) cycle on the 9-point element stencils of k_fevar.cu,
 // (sigma M + tau K(a)) u = r per spectral plane: the colour-ordered Gauss-Seidel sweep from
 // zero, the residual and its restriction by P^T of one level in one launch, and all small
-// levels in another.  (Run colour by colour and level by level, an apply at 127^2 x 130
-// planes took 7 (4 + 2 + 1) launches, 324 us of the ~800 us of a GMRES iteration.)
+// levels in another: at 127^2 x 130 planes 46 + 29 us an apply, where running colour by colour
+// and level by level took 7 (4 + 2 + 1) launches and 324 us of a GMRES iteration's 800.
+// Bound by latency and issue (the planes stay in L2).
 //
 // Colours are c = (i1 & 1) + 2 (i2 & 1).  Two facts keep a level in one array:
 // * After the sweep the equation of a point held when the point was swept, so what is left

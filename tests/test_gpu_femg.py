@@ -47,3 +47,25 @@ def test_rows_too_wide_for_a_strip_agree_with_strips():
     v = S.random_vector((2, n, m1, m1), 6)
     w32, w64 = (_apply(2, m1, n, p, a, v) for p in ("fp32", "fp64"))
     assert float((w32 - w64).abs().max() / w64.abs().max()) <= 1e-5
+
+
+# 3D: the small levels alone (1, 7, 15), one fine level (31: two strips of coarse rows with a
+# remainder), many planes
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-12), ("fp32", 1e-5)])
+@pytest.mark.parametrize("m1,n", [(1, 2), (7, 40), (15, 3), (31, 1), (31, 20)])
+def test_layers_match_oracle(m1, n, precision, tol):
+    a = np.exp(0.4 * S.random_vector((m1 + 2,) * 3, 7))
+    v = S.random_vector((2, n) + (m1,) * 3, 8)
+    tau, alpha = osy.time_step(1.0, n), osy.alpha_weight(1.0, n, 1e-3)
+    ref = opc.apply_Peps_inv(v, n, alpha, 0.3, fe.MGSpatialSolverFE(a, tau))
+    w = _apply(3, m1, n, precision, a, v).cpu().numpy()
+    assert np.abs(w - ref).max() / np.abs(ref).max() <= tol
+
+
+def test_layers_of_several_strips_agree_between_precisions():
+    # 63 rows a layer: strips of 16 row pairs in FP32 and 4 in FP64
+    m1, n = 63, 3
+    a = np.exp(0.4 * S.random_vector((m1 + 2,) * 3, 9))
+    v = S.random_vector((2, n) + (m1,) * 3, 10)
+    w32, w64 = (_apply(3, m1, n, p, a, v) for p in ("fp32", "fp64"))
+    assert float((w32 - w64).abs().max() / w64.abs().max()) <= 1e-5
