@@ -806,20 +806,37 @@ __global__ void __launch_bounds__(kStreamThreads, 1) update_df_kernel(float* Vf,
   }
 }
 
+// The second pass reads the hi planes directly, four consecutive elements of a vector a
+// thread (16-byte loads of 2 KB pieces, several vectors' in flight): 5.8 TB/s over the three
+// kernels at 255^2 x 256, 5.1 with one element a thread.  Bound by HBM.  `len` is even, so the last group may hold two elements: what lies beyond
+// len in the last tile is never used.
+__device__ __forceinline__ float4 load_group(const float* p, bool whole) {
+  float4 v = __ldg(reinterpret_cast<const float4*>(p));
+  if (!whole) v.z = v.w = 0.0f;
+  return v;
+}
+
 // Second pass (re-orthogonalisation, gated): e_c = hi_{i0+c} . x with x the hi plane of
 // the new vector nv (FP32 products of hi planes: the coefficients removed here are ~1e-6).
+// A group's four products are summed before they enter the running sum, whose chain is one
+// addition a group.
 template <int CNT>
 __device__ __forceinline__ void multidot_lp_body(const float* __restrict__ Vf, int nvt, int i0, int nv, size_t len,
                                                  double* __restrict__ partial, int ld) {
   float s[CNT];
 #pragma unroll
   for (int c = 0; c < CNT; ++c) s[c] = 0.0f;
-  const size_t stride = (size_t)gridDim.x * blockDim.x;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < len; e += stride) {
-    const float x = Vf[df_at(nvt, nv, e, 0)];
+  const size_t stride = (size_t)gridDim.x * blockDim.x, groups = (len + 3) / 4;
+  for (size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x; g < groups; g += stride) {
+    const size_t e = 4 * g;
+    const bool whole = e + 4 <= len;
+    const float4 x = load_group(Vf + df_at(nvt, nv, e, 0), whole);
     const float* vb = Vf + df_at(nvt, i0, e, 0);  // vector i0 + c at vb + 2 c kTile
+    float4 v[CNT];
 #pragma unroll
-    for (int c = 0; c < CNT; ++c) s[c] = fmaf(__ldg(vb + (size_t)2 * c * kTile), x, s[c]);
+    for (int c = 0; c < CNT; ++c) v[c] = load_group(vb + (size_t)2 * c * kTile, whole);
+#pragma unroll
+    for (int c = 0; c < CNT; ++c) s[c] += fmaf(v[c].w, x.w, fmaf(v[c].z, x.z, fmaf(v[c].y, x.y, v[c].x * x.x)));
   }
   __shared__ double red[kThreads / 32][CNT];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -863,6 +880,16 @@ __global__ void __launch_bounds__(kThreads) multidot_lp_dyn_kernel(const float* 
   }
 }
 
+constexpr int kLpBatch = 8;  // vectors whose loads are in flight together in the second pass's update
+
+// four (the last group: two) consecutive elements; p is 16-byte aligned
+__device__ __forceinline__ void store_group(float* p, const float (&v)[4], bool whole) {
+  if (whole)
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  else
+    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+}
+
 // Second pass update (gated): vector nv -= sum_i e_i hi_i (FP32 sum of hi planes) in
 // place; partial[b] = block sum of |v|^2.  With jdev: nv = *jdev + 1.
 __global__ void __launch_bounds__(kThreads) update_lp_kernel(float* Vf, int nvt, int nv,
@@ -877,22 +904,42 @@ __global__ void __launch_bounds__(kThreads) update_lp_kernel(float* Vf, int nvt,
   for (int i = threadIdx.x; i < nv; i += blockDim.x) cf[i] = (float)coef[i];
   __syncthreads();
   double acc = 0.0;
-  const size_t stride = (size_t)gridDim.x * blockDim.x;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < len; e += stride) {
+  const size_t stride = (size_t)gridDim.x * blockDim.x, groups = (len + 3) / 4;
+  for (size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x; g < groups; g += stride) {
+    const size_t e = 4 * g;
+    const bool whole = e + 4 <= len;
     float* o = Vf + df_at(nvt, nv, e, 0);
-    float ah = o[0], al = o[kTile];
+    const float4 h4 = *reinterpret_cast<const float4*>(o), l4 = *reinterpret_cast<const float4*>(o + kTile);
     const float* vb = Vf + df_at(nvt, 0, e, 0);  // vector i at vb + 2 i kTile
-    float sf = 0.0f;
-    for (int i = 0; i < nv; ++i) sf = fmaf(cf[i], __ldg(vb + (size_t)2 * i * kTile), sf);
-    const float s2 = __fsub_rn(ah, sf);
-    const float bb = __fsub_rn(s2, ah);
-    al = __fadd_rn(al, __fadd_rn(__fsub_rn(ah, __fsub_rn(s2, bb)), __fsub_rn(neg_f(sf), bb)));
-    ah = s2;
-    df_renorm(ah, al);
-    const double x = f32_to_f64(ah) + f32_to_f64(al);
-    acc = fma(x, x, acc);
-    o[0] = ah;
-    o[kTile] = al;
+    float sf[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    auto add = [&](float c, float4 v) {
+      sf[0] = fmaf(c, v.x, sf[0]);
+      sf[1] = fmaf(c, v.y, sf[1]);
+      sf[2] = fmaf(c, v.z, sf[2]);
+      sf[3] = fmaf(c, v.w, sf[3]);
+    };
+    int i = 0;
+    for (; i + kLpBatch <= nv; i += kLpBatch) {
+      float4 v[kLpBatch];
+#pragma unroll
+      for (int q = 0; q < kLpBatch; ++q) v[q] = load_group(vb + (size_t)2 * (i + q) * kTile, whole);
+#pragma unroll
+      for (int q = 0; q < kLpBatch; ++q) add(cf[i + q], v[q]);
+    }
+    for (; i < nv; ++i) add(cf[i], load_group(vb + (size_t)2 * i * kTile, whole));
+    float hi[4] = {h4.x, h4.y, h4.z, h4.w}, lo[4] = {l4.x, l4.y, l4.z, l4.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float s2 = __fsub_rn(hi[q], sf[q]);
+      const float bb = __fsub_rn(s2, hi[q]);
+      lo[q] = __fadd_rn(lo[q], __fadd_rn(__fsub_rn(hi[q], __fsub_rn(s2, bb)), __fsub_rn(neg_f(sf[q]), bb)));
+      hi[q] = s2;
+      df_renorm(hi[q], lo[q]);
+      const double x = f32_to_f64(hi[q]) + f32_to_f64(lo[q]);
+      if (whole || q < 2) acc = fma(x, x, acc);
+    }
+    store_group(o, hi, whole);
+    store_group(o + kTile, lo, whole);
   }
   __shared__ double red[kThreads / 32];
   acc = warp_sum(acc);
@@ -931,14 +978,18 @@ __global__ void scale_df_kernel(float* Vf, int nvt, int nv, float* vf, size_t le
   if (!(nrm2[0] > 0.0)) return;
   float sh, sl;
   split_f64(1.0 / sqrt(nrm2[0]), sh, sl);
-  const size_t stride = (size_t)gridDim.x * blockDim.x;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < len; e += stride) {
+  const size_t stride = (size_t)gridDim.x * blockDim.x, groups = (len + 3) / 4;
+  for (size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x; g < groups; g += stride) {
+    const size_t e = 4 * g;
+    const bool whole = e + 4 <= len;
     float* o = Vf + df_at(nvt, nv, e, 0);
-    float hi = o[0], lo = o[kTile];
-    df_scale(hi, lo, sh, sl);
-    o[0] = hi;
-    o[kTile] = lo;
-    vf[e] = hi;
+    const float4 h4 = *reinterpret_cast<const float4*>(o), l4 = *reinterpret_cast<const float4*>(o + kTile);
+    float hi[4] = {h4.x, h4.y, h4.z, h4.w}, lo[4] = {l4.x, l4.y, l4.z, l4.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) df_scale(hi[q], lo[q], sh, sl);
+    store_group(o, hi, whole);
+    store_group(o + kTile, lo, whole);
+    store_group(vf + e, hi, whole);
   }
 }
 
@@ -1049,7 +1100,7 @@ template <int CNT>
 cudaError_t multidot_lp_chunk(Launch& L, const float* Vf, int nvt, int i0, int nv, size_t len, double* partial, int ld,
                               const double* gate, unsigned* blocks_out) {
   auto kern = multidot_lp_kernel<CNT>;
-  const unsigned nb = wave_blocks(kern, 0, len);
+  const unsigned nb = wave_blocks(kern, 0, (len + 3) / 4);
   *blocks_out = nb;
   L.begin(KC_REORTH);
   kern<<<nb, kThreads, 0, L.stream>>>(Vf, nvt, i0, nv, len, partial, ld, gate);
@@ -1233,7 +1284,7 @@ cudaError_t launch_update_df(Launch& L, float* Vf, int nvt, int nv, const double
   unsigned nb;
   cudaError_t e;
   if (lp) {
-    nb = wave_blocks(update_lp_kernel, 0, len);
+    nb = wave_blocks(update_lp_kernel, 0, (len + 3) / 4);
     L.begin(KC_REORTH);
     update_lp_kernel<<<nb, kThreads, 0, L.stream>>>(Vf, nvt, nv, coef, len, partial, gate, nullptr);
     e = L.end(KC_REORTH, 0.0, 0.0);
@@ -1266,7 +1317,7 @@ cudaError_t launch_scale_df(Launch& L, float* Vf, int nvt, int nv, float* vf, si
                             const double* gate) {
   const int kc = gate ? KC_REORTH : KC_SCALE;
   L.begin(kc);
-  scale_df_kernel<<<stream_blocks(len), kThreads, 0, L.stream>>>(Vf, nvt, nv, vf, len, nrm2, gate, nullptr);
+  scale_df_kernel<<<stream_blocks((len + 3) / 4), kThreads, 0, L.stream>>>(Vf, nvt, nv, vf, len, nrm2, gate, nullptr);
   return gate ? L.end(kc, 0.0, 0.0) : L.end(kc, 20.0 * len, 1.0 * len);
 }
 
@@ -1280,7 +1331,7 @@ cudaError_t launch_multidot_df_dev(Launch& L, const float* Vf, int nvt, int nv_m
   const int kc = lp ? KC_REORTH : KC_DOT;
   ChunkGrids cg;
   if (lp) {
-    const unsigned nb = wave_blocks(multidot_lp_dyn_kernel, 0, len);
+    const unsigned nb = wave_blocks(multidot_lp_dyn_kernel, 0, (len + 3) / 4);
     cg = one_grid(nb);
     for (int i0 = 0; i0 < nv_max; i0 += kChunk) {
       L.begin(kc);
@@ -1327,7 +1378,7 @@ cudaError_t launch_update_df_dev(Launch& L, float* Vf, int nvt, int nv_max, cons
   cudaError_t e;
   L.begin(kc);
   if (lp) {
-    nb = wave_blocks(update_lp_kernel, 0, len);
+    nb = wave_blocks(update_lp_kernel, 0, (len + 3) / 4);
     update_lp_kernel<<<nb, kThreads, 0, L.stream>>>(Vf, nvt, nv_max, coef, len, partial, gate, jdev);
   } else {
     const size_t stride = round128((size_t)2 * kGroup * kTile * 4 + (size_t)kTile * 8);
@@ -1348,7 +1399,7 @@ cudaError_t launch_update_df_dev(Launch& L, float* Vf, int nvt, int nv_max, cons
 cudaError_t launch_scale_df_dev(Launch& L, float* Vf, int nvt, const int* jdev, float* vf, size_t len,
                                 const double* nrm2, const double* gate) {
   L.begin(KC_REORTH);
-  scale_df_kernel<<<stream_blocks(len), kThreads, 0, L.stream>>>(Vf, nvt, 0, vf, len, nrm2, gate, jdev);
+  scale_df_kernel<<<stream_blocks((len + 3) / 4), kThreads, 0, L.stream>>>(Vf, nvt, 0, vf, len, nrm2, gate, jdev);
   return L.end(KC_REORTH, 0.0, 0.0);
 }
 
