@@ -477,31 +477,38 @@ struct ArnoldiScalars {
   double* inv;   // 1/c
   double* q;     // computed ||w - V d||^2
   double* rho2;  // squared norm after re-orthogonalisation
-  double* flag;  // 1.0 when the step re-orthogonalised
+  double* flag;  // 1.0 when the step re-orthogonalises
+  unsigned* count;  // blocks of a reduction that have finished (zero between launches)
 };
 constexpr int kMaxBlocksPerSM = 8;  // 256-thread blocks: partial-sum buffers hold SMs*8 rows
+// (`prep`: with ww, the reduction also takes the Pythagorean norm; `check`: the update's reduction
+// also decides on re-orthogonalisation)
 // out = V^T w for nv vectors (stride ldv); optionally *ww = ||w||^2; skipped when gate && *gate == 0
 // (gated launches are booked under KC_REORTH with zero bytes; the caller adds them if they ran)
 // lp_reorth: gated (re-orthogonalisation) launches take FP32 products of 20-bit truncations;
 // false keeps FP64 products there too
 cudaError_t launch_multidot(Launch& L, const double* V, size_t ldv, int nv, const double* w, size_t len,
-                            double* partial, double* out, double* ww, const double* gate, bool lp_reorth = true);
+                            double* partial, double* out, double* ww, const double* gate, bool lp_reorth = true,
+                            const ArnoldiScalars* prep = nullptr);
 // v = (v - sum_i coef_i V_i) * (*scale or 1); *q = ||v - sum_i coef_i V_i||^2 (before scaling); gated
 cudaError_t launch_update(Launch& L, const double* V, size_t ldv, int nv, const double* coef, double* v, size_t len,
                           const double* scale, double* partial, double* q, const double* gate, float* vf = nullptr,
-                          bool lp_reorth = true);
-cudaError_t launch_norm2(Launch& L, const double* w, size_t len, double* partial, double* nrm2);
+                          bool lp_reorth = true, const ArnoldiScalars* check = nullptr);
+// *nrm2 = ||w||^2, or ||minuend - w||^2
+cudaError_t launch_norm2(Launch& L, const double* w, size_t len, double* partial, double* nrm2,
+                         const double* minuend = nullptr);
 // v *= 1/sqrt(*nrm2); gated
 cudaError_t launch_scale_by_inv_norm(Launch& L, double* v, size_t len, const double* nrm2, const double* gate,
                                      float* vf = nullptr);
 // y = a*x + b*y (x may be float)
 template <typename Tx>
 cudaError_t launch_axpby(Launch& L, double a, const Tx* x, double b, double* y, size_t len);
-cudaError_t launch_arnoldi_prep(Launch& L, int nv, const double* d, ArnoldiScalars s);
-cudaError_t launch_arnoldi_check(Launch& L, ArnoldiScalars s);
-// column j of H from d (and e after re-orthogonalisation), Givens update, residual estimate
+// column j of H from d (and e after re-orthogonalisation), Givens update, residual estimate;
+// scal[0 .. nscal) is copied to host-mapped memory afterwards.  skip_flagged: a step that asks
+// for re-orthogonalisation is left alone, only its scalars are copied
 cudaError_t launch_givens(Launch& L, int j, int ldh, double* H, double* cs, double* sn, double* gvec, const double* d,
-                          const double* e, ArnoldiScalars s, double* est, const double* ref);
+                          const double* e, ArnoldiScalars s, double* est, const double* ref, bool skip_flagged,
+                          const double* scal, int nscal, double* mapped);
 cudaError_t launch_backsolve(Launch& L, int k, int ldh, const double* H, const double* gvec, double* y);
 template <typename Tz>
 cudaError_t launch_xupdate(Launch& L, const Tz* Z, size_t ldz, int k, const double* y, double* x, size_t len);
@@ -511,18 +518,18 @@ cudaError_t launch_xupdate(Launch& L, const Tz* Z, size_t ldz, int k, const doub
 // can be recorded inside a conditional graph body).
 cudaError_t launch_multidot_dev(Launch& L, const double* V, size_t ldv, int nv_max, const int* jdev,
                                 const double* wbase, size_t wstride, size_t len, double* partial, double* out,
-                                double* ww, const double* gate, bool lp_reorth = true);
+                                double* ww, const double* gate, bool lp_reorth = true,
+                                const ArnoldiScalars* prep = nullptr);
 cudaError_t launch_update_dev(Launch& L, const double* V, size_t ldv, int nv_max, const int* jdev, const double* coef,
                               double* vbase, size_t vstride, size_t len, const double* scale, double* partial,
-                              double* q, const double* gate, float* vf = nullptr, bool lp_reorth = true);
+                              double* q, const double* gate, float* vf = nullptr, bool lp_reorth = true,
+                              const ArnoldiScalars* check = nullptr);
 cudaError_t launch_scale_dev(Launch& L, double* vbase, size_t vstride, const int* jdev, size_t len,
                              const double* nrm2, const double* gate, float* vf = nullptr);
-cudaError_t launch_arnoldi_prep_dev(Launch& L, const int* jdev, const double* d, ArnoldiScalars s);
-cudaError_t launch_givens_dev(Launch& L, const int* jdev, int ldh, double* H, double* cs, double* sn, double* gvec,
-                              const double* d, const double* e, ArnoldiScalars s, double* est, const double* ref);
-// loop control of the captured iteration (sets the WHILE condition; k = iterations done)
-cudaError_t launch_loop_control(Launch& L, int* jdev, int* kdev, const double* est, double rtol, int maxit,
-                                cudaGraphConditionalHandle hc);
+// also the loop control of the captured iteration (sets the WHILE condition; *kdev = iterations done)
+cudaError_t launch_givens_dev(Launch& L, int* jdev, int* kdev, int ldh, double* H, double* cs, double* sn, double* gvec,
+                              const double* d, const double* e, ArnoldiScalars s, double* est, const double* ref,
+                              double rtol, int maxit, cudaGraphConditionalHandle hc);
 cudaError_t launch_loop_start(Launch& L, int* jdev, int* kdev, const double* est, double rtol,
                               cudaGraphConditionalHandle hc);
 cudaError_t launch_backsolve_dev(Launch& L, const int* kdev, int ldh, const double* H, const double* gvec, double* y);
@@ -543,20 +550,22 @@ cudaError_t launch_arnoldi_start(Launch& L, double* gvec, const double* nrm2, do
 // gate != nullptr selects the (gated) second pass on the hi planes.  vf receives the
 // contiguous hi plane (FP32 rounding) of the vector a kernel finishes.
 cudaError_t launch_multidot_df(Launch& L, const float* Vf, int nvt, int nv, const double* w, size_t len,
-                               double* partial, double* out, double* ww, const double* gate, double* err);
+                               double* partial, double* out, double* ww, const double* gate, double* err,
+                               const ArnoldiScalars* prep = nullptr);
 cudaError_t launch_update_df(Launch& L, float* Vf, int nvt, int nv, const double* coef, const double* w, float* vf,
                              size_t len, const double* scale, double* partial, double* q, const double* gate,
-                             double* err);
+                             double* err, const ArnoldiScalars* check = nullptr);
 cudaError_t launch_split_scale(Launch& L, const double* src, float* Vf, int nvt, float* vf, size_t len,
                                const double* nrm2);
 cudaError_t launch_scale_df(Launch& L, float* Vf, int nvt, int nv, float* vf, size_t len, const double* nrm2,
                             const double* gate);
 cudaError_t launch_multidot_df_dev(Launch& L, const float* Vf, int nvt, int nv_max, const int* jdev, const double* w,
                                    size_t len, double* partial, double* out, double* ww, const double* gate,
-                                   double* err);
+                                   double* err, const ArnoldiScalars* prep = nullptr);
 cudaError_t launch_update_df_dev(Launch& L, float* Vf, int nvt, int nv_max, const int* jdev, const double* coef,
                                  const double* w, float* vf, size_t len, const double* scale, double* partial,
-                                 double* q, const double* gate, double* err);
+                                 double* q, const double* gate, double* err,
+                                 const ArnoldiScalars* check = nullptr);
 cudaError_t launch_scale_df_dev(Launch& L, float* Vf, int nvt, const int* jdev, float* vf, size_t len,
                                 const double* nrm2, const double* gate);
 cudaError_t launch_build_rhs(Launch& L, int64_t ms, int n, double tau, double sqrt_gamma, const double* f,

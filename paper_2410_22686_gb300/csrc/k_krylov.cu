@@ -2,11 +2,13 @@
 //
 // One Arnoldi step for the new vector w (stored in place of v_{j+1}):
 //   pass 1  d = V^T w and ||w||^2                       (multidot, one read of V and w)
-//   prep    c = sqrt(||w||^2 - ||d||^2)  (Pythagoras)    (one thread)
+//   prep    c = sqrt(||w||^2 - ||d||^2)  (Pythagoras)    (the last block of the reduction of d)
 //   pass 2  v_{j+1} = (w - V d) / c, q = ||w - V d||^2   (update, one read of V and w, one write)
 //   check   re-orthogonalise if the projection cancelled most of w or Pythagoras is
-//           inaccurate: then pass 1/2 run again on v_{j+1} and it is renormalised
-//           (the gated kernels return at once when the check passed)
+//           inaccurate (in the reduction of q): then pass 1/2 run again on v_{j+1} and it is
+//           renormalised.  The host-driven loop launches that second pass when the scalars
+//           it reads anyway ask for it; captured iterations hold it as gated kernels,
+//           which return at once when the check passed
 //   givens  column j of H = d (+ c e), h_{j+1,j} = c (or c rho); rotations; |g_{j+1}|/ref
 // This is classical Gram-Schmidt with selective re-orthogonalisation: two passes
 // over the basis per iteration in the common case instead of four.
@@ -41,6 +43,35 @@ __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   return v;
+}
+
+// Sums of CNT values over the warp: lane 0 .. of the result hold them.  Each exchange halves
+// the values a lane carries, so the warp issues P + 5 - log2 P - 1 additions (P = CNT rounded up
+// to a power of two) where CNT separate sums issue 5 CNT: on the FP64 unit, a warp's addition
+// every ~18 cycles of an SM, those were a quarter of the FP64 multi-dot at 127^2 x 128 and
+// 6.7 us of every launch of the streamed one.  Returns the sum of value `index` (this lane's);
+// lanes with the same index hold the same sum.
+template <int CNT>
+__device__ __forceinline__ double warp_sums(const double (&v)[CNT], int lane, int& index) {
+  constexpr int P = CNT > 8 ? 16 : CNT > 4 ? 8 : CNT > 2 ? 4 : CNT > 1 ? 2 : 1;
+  double a[P];
+#pragma unroll
+  for (int i = 0; i < P; ++i) a[i] = i < CNT ? v[i < CNT ? i : 0] : 0.0;
+  index = 0;
+  int o = 16;
+#pragma unroll
+  for (int w = P / 2; w >= 1; w >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+    index += up ? w : 0;
+#pragma unroll
+    for (int i = 0; i < w; ++i) {
+      const double send = up ? a[i] : a[i + w];
+      a[i] = (up ? a[i + w] : a[i]) + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  double t = a[0];
+  for (; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
 }
 
 __device__ __forceinline__ bool gated_off(const double* gate) { return gate && gate[0] == 0.0; }
@@ -88,10 +119,10 @@ __device__ __forceinline__ void multidot_body(const double* __restrict__ V, size
   }
   __shared__ double red[kThreads / 32][CNT + 1];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int c = 0; c < CNT; ++c) {
-    const double v = warp_sum(acc[c]);
-    if (lane == 0) red[wid][c] = v;
+  {
+    int c;
+    const double v = warp_sums<CNT>(acc, lane, c);
+    if (c < CNT) red[wid][c] = v;
   }
   if (WITH_NORM) {
     const double v = warp_sum(ww);
@@ -144,15 +175,57 @@ struct ChunkGrids {
   unsigned nb[kMaxChunks];
 };
 
+// What follows a reduction in the same launch (by the block that finishes last).
+enum ReduceThen { kThenNothing = 0, kThenPrep = 1, kThenCheck = 2 };
+
+// c = sqrt(||w||^2 - ||d||^2) when that is safely positive, else 1 (and force
+// re-orthogonalisation); one warp
+__device__ __forceinline__ void arnoldi_prep(int nv, const double* d, const ArnoldiScalars& s) {
+  const int lane = threadIdx.x & 31;
+  double dd = 0.0;
+  for (int i = lane; i < nv; i += 32) {
+    const double v = __ldcg(d + i);
+    dd = fma(v, v, dd);
+  }
+  dd = warp_sum(dd);
+  if (lane != 0) return;
+  const double ww = __ldcg(s.ww);
+  const double r = ww - dd;
+  if (r > 1e-12 * ww && r > 0.0) {
+    const double c = sqrt(r);
+    s.c[0] = c;
+    s.inv[0] = 1.0 / c;
+    s.flag[0] = 0.0;
+  } else {
+    s.c[0] = 1.0;
+    s.inv[0] = 1.0;
+    s.flag[0] = 1.0;
+  }
+}
+
+// re-orthogonalise when ||w - V d||^2 < 1e-10 ||w||^2 (one pass then leaves a loss
+// of orthogonality of about eps ||w|| / ||w - V d|| > 1e-11) or when the Pythagorean
+// norm disagrees with the computed one by more than 1e-6 (relative, squared).  With
+// a strong preconditioner A P^{-1} v_j is close to v_j, so strong cancellation is the
+// normal case and a tighter trigger would re-orthogonalise in many iterations.
+__device__ __forceinline__ void arnoldi_check(double q, const ArnoldiScalars& s) {
+  if (s.flag[0] != 0.0) return;
+  const double ww = s.ww[0], c2 = s.c[0] * s.c[0];
+  const bool bad = !(q >= 1e-10 * ww) || !(fabs(q - c2) <= 1e-6 * q);
+  s.flag[0] = bad ? 1.0 : 0.0;
+}
+
 // out[i] = sum_b partial[b*ld + i] for i < nout (column nout goes to *extra), in a
 // fixed order; one block per column
 // With jdev != nullptr: nout = *jdev + 1, the grid covers the largest count, blocks
 // beyond nout exit, and the last block reduces the extra column ld - 1.
+// then = kThenPrep: the block that finishes last (a counter it sets back to zero) takes the
+// Pythagorean norm of out[0 .. nout) and *extra; kThenCheck (one block): the check of out[0].
 __global__ void __launch_bounds__(kThreads) reduce_partials_kernel(const double* __restrict__ partial, ChunkGrids cg,
-                                                                   int ld, double* __restrict__ out,
-                                                                   double* __restrict__ extra, int nout,
+                                                                   int ld, double* out, double* extra, int nout,
                                                                    const double* __restrict__ gate,
-                                                                   const int* __restrict__ jdev) {
+                                                                   const int* __restrict__ jdev, int then,
+                                                                   ArnoldiScalars as) {
   if (gated_off(gate)) return;
   int i = blockIdx.x;
   if (jdev) {
@@ -167,6 +240,7 @@ __global__ void __launch_bounds__(kThreads) reduce_partials_kernel(const double*
   double s = 0.0;
   for (int b = threadIdx.x; b < nblocks; b += blockDim.x) s += partial[(size_t)b * ld + i];
   __shared__ double red[kThreads / 32];
+  __shared__ bool last;
   s = warp_sum(s);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
@@ -177,6 +251,20 @@ __global__ void __launch_bounds__(kThreads) reduce_partials_kernel(const double*
       out[i] = t;
     else
       extra[0] = t;
+    last = false;
+    if (then == kThenPrep) {
+      __threadfence();
+      last = atomicAdd(as.count, 1u) == (unsigned)nout;  // nout columns and the norm's
+      if (last) *as.count = 0u;
+    } else if (then == kThenCheck) {
+      arnoldi_check(t, as);
+    }
+  }
+  if (then != kThenPrep) return;
+  __syncthreads();
+  if (last && threadIdx.x < 32) {
+    __threadfence();
+    arnoldi_prep(nout, out, as);
   }
 }
 
@@ -235,11 +323,16 @@ __global__ void __launch_bounds__(kThreads) update_kernel(const double* __restri
   }
 }
 
-__global__ void __launch_bounds__(kThreads) norm2_kernel(const double* __restrict__ w, size_t len,
+// partial[b] = block sum of w^2, or of (minuend - w)^2
+__global__ void __launch_bounds__(kThreads) norm2_kernel(const double* __restrict__ w,
+                                                         const double* __restrict__ minuend, size_t len,
                                                          double* __restrict__ partial) {
   double acc = 0.0;
   const size_t stride = (size_t)gridDim.x * blockDim.x;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < len; e += stride) acc = fma(w[e], w[e], acc);
+  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < len; e += stride) {
+    const double x = minuend ? minuend[e] - w[e] : w[e];
+    acc = fma(x, x, acc);
+  }
   __shared__ double red[kThreads / 32];
   acc = warp_sum(acc);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
@@ -274,92 +367,109 @@ __global__ void axpby_kernel(double a, const Tx* __restrict__ x, double b, doubl
     y[e] = (b == 0.0) ? a * cvt<double>(x[e]) : fma(a, cvt<double>(x[e]), b * y[e]);
 }
 
-// c = sqrt(||w||^2 - ||d||^2) when that is safely positive, else 1 (and force re-orthogonalisation)
-__global__ void arnoldi_prep_kernel(int nv, const double* d, ArnoldiScalars s, const int* jdev) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  if (jdev) nv = *jdev + 1;
-  double dd = 0.0;
-  for (int i = 0; i < nv; ++i) dd = fma(d[i], d[i], dd);
-  const double ww = s.ww[0];
-  const double r = ww - dd;
-  if (r > 1e-12 * ww && r > 0.0) {
-    s.c[0] = sqrt(r);
-    s.inv[0] = 1.0 / s.c[0];
-    s.flag[0] = 0.0;
-  } else {
-    s.c[0] = 1.0;
-    s.inv[0] = 1.0;
-    s.flag[0] = 1.0;
-  }
-}
-
-// re-orthogonalise when ||w - V d||^2 < 1e-10 ||w||^2 (one pass then leaves a loss
-// of orthogonality of about eps ||w|| / ||w - V d|| > 1e-11) or when the Pythagorean
-// norm disagrees with the computed one by more than 1e-6 (relative, squared).  With
-// a strong preconditioner A P^{-1} v_j is close to v_j, so strong cancellation is the
-// normal case and a tighter trigger would re-orthogonalise in many iterations.
-__global__ void arnoldi_check_kernel(ArnoldiScalars s) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  if (s.flag[0] != 0.0) return;
-  const double q = s.q[0], ww = s.ww[0], c2 = s.c[0] * s.c[0];
-  const bool bad = !(q >= 1e-10 * ww) || !(fabs(q - c2) <= 1e-6 * q);
-  s.flag[0] = bad ? 1.0 : 0.0;
-}
+// What the Givens step hands on: the scalars the host reads (mapped memory), or the loop
+// condition of a captured iteration (jdev, kdev: Arnoldi index and iterations done).
+struct GivensOut {
+  double* mapped;         // host-mapped copy of scal[0 .. nscal), or null
+  const double* scal;
+  int nscal;
+  int *jdev, *kdev;       // captured iterations, else null
+  double rtol;
+  int maxit;
+  cudaGraphConditionalHandle hc;
+};
 
 // Column j of H and its Givens rotation; est = |g_{j+1}| / ref.
 //   no re-orthogonalisation:  w = V d + c v_{j+1}
 //   re-orthogonalisation:     w = V (d + c e) + c rho v_{j+1},  rho^2 = s.rho2
+// With skip_flagged a step whose check asked for re-orthogonalisation is left alone (its
+// second pass has not run yet); the host sees the flag.
 __global__ void givens_kernel(int j, int ldh, double* H, double* cs, double* sn, double* g, const double* d,
-                              const double* e, ArnoldiScalars s, double* est, const double* ref, const int* jdev) {
+                              const double* e, ArnoldiScalars s, double* est, const double* ref, const int* jdev,
+                              bool skip_flagged, GivensOut out) {
   if (blockIdx.x != 0) return;
   if (jdev) j = *jdev;
   // the warp stages the column and the rotations in shared memory; one thread then
-  // applies the j sequential rotations without waiting on global memory
+  // applies the j sequential rotations, the running entry in a register
   __shared__ double cl[1026], sc[1024], ss[1024];
   double* col = H + (size_t)j * ldh;
   const bool re = s.flag[0] != 0.0;
   const double c = s.c[0];
-  for (int i = threadIdx.x; i <= j; i += blockDim.x) {
-    cl[i] = re ? fma(c, e[i], d[i]) : d[i];
-    if (i < j) {
-      sc[i] = cs[i];
-      ss[i] = sn[i];
+  if (!(re && skip_flagged)) {
+    for (int i = threadIdx.x; i <= j; i += blockDim.x) {
+      const double di = d[i];
+      cl[i] = re ? fma(c, e[i], di) : di;
+      if (i < j) {
+        sc[i] = cs[i];
+        ss[i] = sn[i];
+      }
     }
+    const double gj = threadIdx.x == 0 ? g[j] : 0.0, rf = threadIdx.x == 0 ? ref[0] : 1.0;
+    __syncwarp();
+    if (threadIdx.x == 0) {
+      const double b = re ? c * sqrt(s.rho2[0]) : c;
+      double a = cl[0];
+#pragma unroll 4
+      for (int i = 0; i < j; ++i) {
+        const double nx = cl[i + 1], ci = sc[i], si = ss[i];
+        cl[i] = fma(si, nx, ci * a);
+        a = fma(ci, nx, -si * a);
+      }
+      double cr = 1.0, sr = 0.0, r = a;
+      if (b != 0.0) {
+        r = hypot(a, b);
+        cr = a / r;
+        sr = b / r;
+      }
+      cs[j] = cr;
+      sn[j] = sr;
+      cl[j] = r;
+      cl[j + 1] = 0.0;
+      g[j + 1] = -sr * gj;
+      g[j] = cr * gj;
+      est[0] = fabs(sr * gj) / rf;
+    }
+    __syncwarp();
+    for (int i = threadIdx.x; i <= j + 1; i += blockDim.x) col[i] = cl[i];
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    cl[j + 1] = re ? c * sqrt(s.rho2[0]) : c;
-    for (int i = 0; i < j; ++i) {
-      const double t = sc[i] * cl[i] + ss[i] * cl[i + 1];
-      cl[i + 1] = -ss[i] * cl[i] + sc[i] * cl[i + 1];
-      cl[i] = t;
-    }
-    const double a = cl[j], b = cl[j + 1];
-    double cr = 1.0, sr = 0.0, r = a;
-    if (b != 0.0) {
-      r = hypot(a, b);
-      cr = a / r;
-      sr = b / r;
-    }
-    cs[j] = cr;
-    sn[j] = sr;
-    cl[j] = r;
-    cl[j + 1] = 0.0;
-    g[j + 1] = -sr * g[j];
-    g[j] = cr * g[j];
-    est[0] = fabs(g[j + 1]) / ref[0];
+  if (out.mapped) {
+    __syncwarp();
+    for (int i = threadIdx.x; i < out.nscal; i += blockDim.x) out.mapped[i] = out.scal[i];
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i <= j + 1; i += blockDim.x) col[i] = cl[i];
+  if (out.jdev && threadIdx.x == 0) {
+    // continue (condition 1) while the estimate is finite, above rtol and j + 1 < maxit
+    const double ev = est[0];
+    const bool cont = isfinite(ev) && ev > out.rtol && j + 1 < out.maxit;
+    *out.kdev = j + 1;
+    if (cont) *out.jdev = j + 1;
+    cudaGraphSetConditional(out.hc, cont ? 1u : 0u);
+  }
 }
 
-__global__ void backsolve_kernel(int k, int ldh, const double* H, const double* g, double* y, const int* kdev) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// y = R^{-1} g by columns: once y_i is known every lane of the first warp updates its rows.
+// The columns of up to kBackStage steps are staged in shared memory first (each one waits for
+// the one before it, so their loads would not overlap): one thread by rows took 31 us for
+// 18 columns, this 5.
+constexpr int kBackStage = 72, kBackThreads = 256;
+__global__ void __launch_bounds__(kBackThreads) backsolve_kernel(int k, int ldh, const double* H, const double* g,
+                                                                 double* y, const int* kdev) {
+  if (blockIdx.x != 0) return;
   if (kdev) k = *kdev;
+  __shared__ double t[1024], R[kBackStage * (kBackStage + 1) / 2];
+  const bool staged = k <= kBackStage;
+  if (staged)
+    for (int i = threadIdx.x >> 5; i < k; i += kBackThreads / 32)
+      for (int q = threadIdx.x & 31; q <= i; q += 32) R[i * (i + 1) / 2 + q] = H[(size_t)i * ldh + q];
+  for (int i = threadIdx.x; i < k; i += kBackThreads) t[i] = g[i];
+  __syncthreads();
+  const int lane = threadIdx.x;
+  if (lane >= 32) return;
   for (int i = k - 1; i >= 0; --i) {
-    double s = g[i];
-    for (int q = i + 1; q < k; ++q) s -= H[(size_t)q * ldh + i] * y[q];
-    y[i] = s / H[(size_t)i * ldh + i];
+    const double* col = staged ? R + i * (i + 1) / 2 : H + (size_t)i * ldh;
+    const double yi = t[i] / col[i];
+    if (lane == 0) y[i] = yi;
+    for (int q = lane; q < i; q += 32) t[q] = fma(-col[q], yi, t[q]);
+    __syncwarp();
   }
 }
 
@@ -412,19 +522,6 @@ __global__ void arnoldi_start_kernel(double* g, const double* nrm2, double* est,
   g[0] = beta;
   if (set_ref) ref[0] = beta;
   est[0] = beta / ref[0];
-}
-
-// Loop control of a graph-captured FGMRES iteration: k = j + 1 iterations are done;
-// continue (condition 1) while the estimate is finite, above rtol and j + 1 < maxit.
-__global__ void loop_control_kernel(int* jdev, int* kdev, const double* est, double rtol, int maxit,
-                                    cudaGraphConditionalHandle hc) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const int j = *jdev;
-  const double e = est[0];
-  const bool cont = isfinite(e) && e > rtol && j + 1 < maxit;
-  *kdev = j + 1;
-  if (cont) *jdev = j + 1;
-  cudaGraphSetConditional(hc, cont ? 1u : 0u);
 }
 
 // Before the loop: j = k = 0, and enter the loop only when the initial estimate is
@@ -645,10 +742,13 @@ __device__ __forceinline__ void multidot_df_stream(const float* __restrict__ Vf,
   stream_items(mine, S, stage_stride, issue, consume, err);
   __shared__ double red[kStreamThreads / 32][CNT + 1];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  {
+    double t[CNT];
 #pragma unroll
-  for (int c = 0; c < CNT; ++c) {
-    const double v = warp_sum(f32_to_f64(s[c]) + f32_to_f64(er[c]));
-    if (lane == 0) red[wid][c] = v;
+    for (int c = 0; c < CNT; ++c) t[c] = f32_to_f64(s[c]) + f32_to_f64(er[c]);
+    int c;
+    const double v = warp_sums<CNT>(t, lane, c);
+    if (c < CNT) red[wid][c] = v;
   }
   if (WITH_NORM) {
     const double v = warp_sum(ww);
@@ -840,10 +940,13 @@ __device__ __forceinline__ void multidot_lp_body(const float* __restrict__ Vf, i
   }
   __shared__ double red[kThreads / 32][CNT];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  {
+    double t[CNT];
 #pragma unroll
-  for (int c = 0; c < CNT; ++c) {
-    const double v = warp_sum(f32_to_f64(s[c]));
-    if (lane == 0) red[wid][c] = v;
+    for (int c = 0; c < CNT; ++c) t[c] = f32_to_f64(s[c]);
+    int c;
+    const double v = warp_sums<CNT>(t, lane, c);
+    if (c < CNT) red[wid][c] = v;
   }
   __syncthreads();
   if (threadIdx.x < CNT) {
@@ -1123,7 +1226,8 @@ cudaError_t multidot_lp_dispatch(int cnt, Launch& L, const float* Vf, int nvt, i
 }  // namespace
 
 cudaError_t launch_multidot(Launch& L, const double* V, size_t ldv, int nv, const double* w, size_t len,
-                            double* partial, double* out, double* ww, const double* gate, bool lp_reorth) {
+                            double* partial, double* out, double* ww, const double* gate, bool lp_reorth,
+                            const ArnoldiScalars* prep) {
   if (nv < 1 || nv > kChunk * kMaxChunks) return cudaErrorInvalidValue;
   const int ld = nv + 1;
   ChunkGrids cg = one_grid(1);
@@ -1141,13 +1245,15 @@ cudaError_t launch_multidot(Launch& L, const double* V, size_t ldv, int nv, cons
   const int ncols = nv + (ww ? 1 : 0);
   const int kc = gate ? KC_REORTH : KC_REDUCE;
   L.begin(kc);
-  reduce_partials_kernel<<<ncols, kThreads, 0, L.stream>>>(partial, cg, ld, out, ww, nv, gate, nullptr);
+  reduce_partials_kernel<<<ncols, kThreads, 0, L.stream>>>(partial, cg, ld, out, ww, nv, gate, nullptr,
+                                                          prep && ww ? kThenPrep : kThenNothing,
+                                                          prep ? *prep : ArnoldiScalars{});
   return gate ? L.end(kc, 0.0, 0.0) : L.end(kc, 8.0 * nb_sum, nb_sum);
 }
 
 cudaError_t launch_update(Launch& L, const double* V, size_t ldv, int nv, const double* coef, double* v, size_t len,
                           const double* scale, double* partial, double* q, const double* gate, float* vf,
-                          bool lp_reorth) {
+                          bool lp_reorth, const ArnoldiScalars* check) {
   const size_t smem = sizeof(double) * (nv > 0 ? nv : 1);
   auto kern = (gate && lp_reorth) ? update_kernel<true> : update_kernel<false>;  // gated: re-orthogonalisation
   const unsigned nb = wave_blocks(kern, smem, len);
@@ -1159,19 +1265,22 @@ cudaError_t launch_update(Launch& L, const double* V, size_t ldv, int nv, const 
   if (e != cudaSuccess) return e;
   const int kr = gate ? KC_REORTH : KC_REDUCE;
   L.begin(kr);
-  reduce_partials_kernel<<<1, kThreads, 0, L.stream>>>(partial, one_grid(nb), 1, q, q, 1, gate, nullptr);
+  reduce_partials_kernel<<<1, kThreads, 0, L.stream>>>(partial, one_grid(nb), 1, q, q, 1, gate, nullptr,
+                                                       check ? kThenCheck : kThenNothing,
+                                                       check ? *check : ArnoldiScalars{});
   return gate ? L.end(kr, 0.0, 0.0) : L.end(kr, 8.0 * nb, 1.0 * nb);
 }
 
-cudaError_t launch_norm2(Launch& L, const double* w, size_t len, double* partial, double* nrm2) {
+cudaError_t launch_norm2(Launch& L, const double* w, size_t len, double* partial, double* nrm2,
+                         const double* minuend) {
   const unsigned nb = wave_blocks(norm2_kernel, 0, len);
   L.begin(KC_DOT);
-  norm2_kernel<<<nb, kThreads, 0, L.stream>>>(w, len, partial);
-  cudaError_t e = L.end(KC_DOT, 8.0 * len, 2.0 * len);
+  norm2_kernel<<<nb, kThreads, 0, L.stream>>>(w, minuend, len, partial);
+  cudaError_t e = L.end(KC_DOT, (minuend ? 16.0 : 8.0) * len, 2.0 * len);
   if (e != cudaSuccess) return e;
   L.begin(KC_REDUCE);
   reduce_partials_kernel<<<1, kThreads, 0, L.stream>>>(partial, one_grid(nb), 1, nrm2, nrm2, 1, nullptr,
-                                                       nullptr);
+                                                       nullptr, kThenNothing, ArnoldiScalars{});
   return L.end(KC_REDUCE, 8.0 * nb, 1.0 * nb);
 }
 
@@ -1192,28 +1301,18 @@ cudaError_t launch_axpby(Launch& L, double a, const Tx* x, double b, double* y, 
 template cudaError_t launch_axpby<double>(Launch&, double, const double*, double, double*, size_t);
 template cudaError_t launch_axpby<float>(Launch&, double, const float*, double, double*, size_t);
 
-cudaError_t launch_arnoldi_prep(Launch& L, int nv, const double* d, ArnoldiScalars s) {
-  L.begin(KC_GIVENS);
-  arnoldi_prep_kernel<<<1, 32, 0, L.stream>>>(nv, d, s, nullptr);
-  return L.end(KC_GIVENS, 0.0, 2.0 * nv);
-}
-
-cudaError_t launch_arnoldi_check(Launch& L, ArnoldiScalars s) {
-  L.begin(KC_GIVENS);
-  arnoldi_check_kernel<<<1, 32, 0, L.stream>>>(s);
-  return L.end(KC_GIVENS, 0.0, 4.0);
-}
-
 cudaError_t launch_givens(Launch& L, int j, int ldh, double* H, double* cs, double* sn, double* gvec, const double* d,
-                          const double* e, ArnoldiScalars s, double* est, const double* ref) {
+                          const double* e, ArnoldiScalars s, double* est, const double* ref, bool skip_flagged,
+                          const double* scal, int nscal, double* mapped) {
+  GivensOut out{mapped, scal, nscal, nullptr, nullptr, 0.0, 0, cudaGraphConditionalHandle{}};
   L.begin(KC_GIVENS);
-  givens_kernel<<<1, 32, 0, L.stream>>>(j, ldh, H, cs, sn, gvec, d, e, s, est, ref, nullptr);
+  givens_kernel<<<1, 32, 0, L.stream>>>(j, ldh, H, cs, sn, gvec, d, e, s, est, ref, nullptr, skip_flagged, out);
   return L.end(KC_GIVENS, 0.0, 10.0 * (j + 1));
 }
 
 cudaError_t launch_backsolve(Launch& L, int k, int ldh, const double* H, const double* gvec, double* y) {
   L.begin(KC_GIVENS);
-  backsolve_kernel<<<1, 32, 0, L.stream>>>(k, ldh, H, gvec, y, nullptr);
+  backsolve_kernel<<<1, kBackThreads, 0, L.stream>>>(k, ldh, H, gvec, y, nullptr);
   return L.end(KC_GIVENS, 0.0, 1.0 * k * k);
 }
 
@@ -1238,7 +1337,8 @@ cudaError_t launch_arnoldi_start(Launch& L, double* gvec, const double* nrm2, do
 // ---------------------------------------------------------------------------
 // double-float basis in the tiled layout (df_at); vector nv is the new one
 cudaError_t launch_multidot_df(Launch& L, const float* Vf, int nvt, int nv, const double* w, size_t len,
-                               double* partial, double* out, double* ww, const double* gate, double* err) {
+                               double* partial, double* out, double* ww, const double* gate, double* err,
+                               const ArnoldiScalars* prep) {
   if (nv < 1 || nv >= nvt || nv > kChunk * kMaxChunks) return cudaErrorInvalidValue;
   if (len & 1) return cudaErrorInvalidValue;  // the streamed tiles need an even length
   const bool lp = gate != nullptr;  // gated launches are the re-orthogonalisation pass
@@ -1271,13 +1371,14 @@ cudaError_t launch_multidot_df(Launch& L, const float* Vf, int nvt, int nv, cons
   const int kc = lp ? KC_REORTH : KC_REDUCE;
   L.begin(kc);
   reduce_partials_kernel<<<ncols, kThreads, 0, L.stream>>>(partial, cg, ld, out, lp ? nullptr : ww, nv, gate,
-                                                          nullptr);
+                                                          nullptr, prep && ww && !lp ? kThenPrep : kThenNothing,
+                                                          prep ? *prep : ArnoldiScalars{});
   return lp ? L.end(kc, 0.0, 0.0) : L.end(kc, 8.0 * nb_sum, nb_sum);
 }
 
 cudaError_t launch_update_df(Launch& L, float* Vf, int nvt, int nv, const double* coef, const double* w, float* vf,
                              size_t len, const double* scale, double* partial, double* q, const double* gate,
-                             double* err) {
+                             double* err, const ArnoldiScalars* check) {
   if (nv < 1 || nv >= nvt || nv > 1024) return cudaErrorInvalidValue;
   if (len & 1) return cudaErrorInvalidValue;
   const bool lp = gate != nullptr;
@@ -1302,7 +1403,9 @@ cudaError_t launch_update_df(Launch& L, float* Vf, int nvt, int nv, const double
   if (e != cudaSuccess) return e;
   const int kr = lp ? KC_REORTH : KC_REDUCE;
   L.begin(kr);
-  reduce_partials_kernel<<<1, kThreads, 0, L.stream>>>(partial, one_grid(nb), 1, q, q, 1, gate, nullptr);
+  reduce_partials_kernel<<<1, kThreads, 0, L.stream>>>(partial, one_grid(nb), 1, q, q, 1, gate, nullptr,
+                                                       check ? kThenCheck : kThenNothing,
+                                                       check ? *check : ArnoldiScalars{});
   return lp ? L.end(kr, 0.0, 0.0) : L.end(kr, 8.0 * nb, 1.0 * nb);
 }
 
@@ -1323,7 +1426,7 @@ cudaError_t launch_scale_df(Launch& L, float* Vf, int nvt, int nv, float* vf, si
 
 cudaError_t launch_multidot_df_dev(Launch& L, const float* Vf, int nvt, int nv_max, const int* jdev, const double* w,
                                    size_t len, double* partial, double* out, double* ww, const double* gate,
-                                   double* err) {
+                                   double* err, const ArnoldiScalars* prep) {
   if (nv_max < 1 || nv_max >= nvt || nv_max > kChunk * kMaxChunks) return cudaErrorInvalidValue;
   if (len & 1) return cudaErrorInvalidValue;
   const bool lp = gate != nullptr;
@@ -1363,13 +1466,16 @@ cudaError_t launch_multidot_df_dev(Launch& L, const float* Vf, int nvt, int nv_m
   L.begin(kc);
   reduce_partials_kernel<<<nv_max + (ww && !lp ? 1 : 0), kThreads, 0, L.stream>>>(partial, cg, ld, out,
                                                                                  lp ? nullptr : ww, nv_max, gate,
-                                                                                 jdev);
+                                                                                 jdev,
+                                                                                 prep && ww && !lp ? kThenPrep
+                                                                                                   : kThenNothing,
+                                                                                 prep ? *prep : ArnoldiScalars{});
   return L.end(kc, 0.0, 0.0);
 }
 
 cudaError_t launch_update_df_dev(Launch& L, float* Vf, int nvt, int nv_max, const int* jdev, const double* coef,
                                  const double* w, float* vf, size_t len, const double* scale, double* partial,
-                                 double* q, const double* gate, double* err) {
+                                 double* q, const double* gate, double* err, const ArnoldiScalars* check) {
   if (nv_max < 1 || nv_max >= nvt || nv_max > 1024) return cudaErrorInvalidValue;
   if (len & 1) return cudaErrorInvalidValue;
   const bool lp = gate != nullptr;
@@ -1392,7 +1498,9 @@ cudaError_t launch_update_df_dev(Launch& L, float* Vf, int nvt, int nv_max, cons
   e = L.end(kc, 0.0, 0.0);
   if (e != cudaSuccess) return e;
   L.begin(kc);
-  reduce_partials_kernel<<<1, kThreads, 0, L.stream>>>(partial, one_grid(nb), 1, q, q, 1, gate, nullptr);
+  reduce_partials_kernel<<<1, kThreads, 0, L.stream>>>(partial, one_grid(nb), 1, q, q, 1, gate, nullptr,
+                                                       check ? kThenCheck : kThenNothing,
+                                                       check ? *check : ArnoldiScalars{});
   return L.end(kc, 0.0, 0.0);
 }
 
@@ -1408,7 +1516,7 @@ cudaError_t launch_scale_df_dev(Launch& L, float* Vf, int nvt, const int* jdev, 
 // index, which the kernels read from `jdev`, so one captured iteration serves all
 cudaError_t launch_multidot_dev(Launch& L, const double* V, size_t ldv, int nv_max, const int* jdev,
                                 const double* wbase, size_t wstride, size_t len, double* partial, double* out,
-                                double* ww, const double* gate, bool lp_reorth) {
+                                double* ww, const double* gate, bool lp_reorth, const ArnoldiScalars* prep) {
   if (nv_max < 1 || nv_max > kChunk * kMaxChunks) return cudaErrorInvalidValue;
   const int ld = nv_max + 1;
   // gated launches are the re-orthogonalisation pass: FP32 products (see the file header)
@@ -1431,13 +1539,15 @@ cudaError_t launch_multidot_dev(Launch& L, const double* V, size_t ldv, int nv_m
   }
   L.begin(kc);
   reduce_partials_kernel<<<nv_max + (ww ? 1 : 0), kThreads, 0, L.stream>>>(partial, cg, ld, out, ww, nv_max, gate,
-                                                                          jdev);
+                                                                          jdev, prep && ww ? kThenPrep : kThenNothing,
+                                                                          prep ? *prep : ArnoldiScalars{});
   return L.end(kc, 0.0, 0.0);
 }
 
 cudaError_t launch_update_dev(Launch& L, const double* V, size_t ldv, int nv_max, const int* jdev, const double* coef,
                               double* vbase, size_t vstride, size_t len, const double* scale, double* partial,
-                              double* q, const double* gate, float* vf, bool lp_reorth) {
+                              double* q, const double* gate, float* vf, bool lp_reorth,
+                              const ArnoldiScalars* check) {
   const size_t smem = sizeof(double) * nv_max;
   auto kern = (gate && lp_reorth) ? update_kernel<true> : update_kernel<false>;  // gated: re-orthogonalisation
   const unsigned nb = wave_blocks(kern, smem, len);
@@ -1448,7 +1558,9 @@ cudaError_t launch_update_dev(Launch& L, const double* V, size_t ldv, int nv_max
   cudaError_t e = L.end(kc, 0.0, 0.0);
   if (e != cudaSuccess) return e;
   L.begin(kc);
-  reduce_partials_kernel<<<1, kThreads, 0, L.stream>>>(partial, one_grid(nb), 1, q, q, 1, gate, nullptr);
+  reduce_partials_kernel<<<1, kThreads, 0, L.stream>>>(partial, one_grid(nb), 1, q, q, 1, gate, nullptr,
+                                                       check ? kThenCheck : kThenNothing,
+                                                       check ? *check : ArnoldiScalars{});
   return L.end(kc, 0.0, 0.0);
 }
 
@@ -1459,23 +1571,12 @@ cudaError_t launch_scale_dev(Launch& L, double* vbase, size_t vstride, const int
   return L.end(KC_REORTH, 0.0, 0.0);
 }
 
-cudaError_t launch_arnoldi_prep_dev(Launch& L, const int* jdev, const double* d, ArnoldiScalars s) {
+cudaError_t launch_givens_dev(Launch& L, int* jdev, int* kdev, int ldh, double* H, double* cs, double* sn, double* gvec,
+                              const double* d, const double* e, ArnoldiScalars s, double* est, const double* ref,
+                              double rtol, int maxit, cudaGraphConditionalHandle hc) {
+  GivensOut out{nullptr, nullptr, 0, jdev, kdev, rtol, maxit, hc};
   L.begin(KC_GIVENS);
-  arnoldi_prep_kernel<<<1, 32, 0, L.stream>>>(0, d, s, jdev);
-  return L.end(KC_GIVENS, 0.0, 0.0);
-}
-
-cudaError_t launch_givens_dev(Launch& L, const int* jdev, int ldh, double* H, double* cs, double* sn, double* gvec,
-                              const double* d, const double* e, ArnoldiScalars s, double* est, const double* ref) {
-  L.begin(KC_GIVENS);
-  givens_kernel<<<1, 32, 0, L.stream>>>(0, ldh, H, cs, sn, gvec, d, e, s, est, ref, jdev);
-  return L.end(KC_GIVENS, 0.0, 0.0);
-}
-
-cudaError_t launch_loop_control(Launch& L, int* jdev, int* kdev, const double* est, double rtol, int maxit,
-                                cudaGraphConditionalHandle hc) {
-  L.begin(KC_GIVENS);
-  loop_control_kernel<<<1, 32, 0, L.stream>>>(jdev, kdev, est, rtol, maxit, hc);
+  givens_kernel<<<1, 32, 0, L.stream>>>(0, ldh, H, cs, sn, gvec, d, e, s, est, ref, jdev, false, out);
   return L.end(KC_GIVENS, 0.0, 0.0);
 }
 
@@ -1488,7 +1589,7 @@ cudaError_t launch_loop_start(Launch& L, int* jdev, int* kdev, const double* est
 
 cudaError_t launch_backsolve_dev(Launch& L, const int* kdev, int ldh, const double* H, const double* gvec, double* y) {
   L.begin(KC_GIVENS);
-  backsolve_kernel<<<1, 32, 0, L.stream>>>(0, ldh, H, gvec, y, kdev);
+  backsolve_kernel<<<1, kBackThreads, 0, L.stream>>>(0, ldh, H, gvec, y, kdev);
   return L.end(KC_GIVENS, 0.0, 0.0);
 }
 
