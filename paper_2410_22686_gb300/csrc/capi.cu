@@ -186,7 +186,7 @@ struct pc_handle {
   // time FFT tables
   double* dpow64 = nullptr;  // eps^{j/n}
   float* dpow32 = nullptr;
-  double* dinv64 = nullptr;  // eps^{-j/n}
+  double* dinv64 = nullptr;  // eps^{-j/n} / (2n)
   float* dinv32 = nullptr;
   double2* tw64 = nullptr;
   float2* tw32 = nullptr;
@@ -768,7 +768,7 @@ static int setup_impl(const pc_params* p, const double* a_nodes, void* krylov, s
     std::vector<double> dp(n), di(n), twr(n), twi(n);
     for (int j = 0; j < n; ++j) {
       dp[j] = std::pow(p->eps, (double)j / n);
-      di[j] = std::pow(p->eps, -(double)j / n);
+      di[j] = std::pow(p->eps, -(double)j / n) / (2.0 * n);
     }
     for (int k = 0; k < n; ++k) {
       const double th = 2.0 * M_PI * (double)k / n;
@@ -1285,7 +1285,6 @@ static FineCorrection<TU> fine_correction(const pc_handle* h) {
   if (h->spatial == PC_SPATIAL_FST || h->lex || h->coarse_l0 < 1 || h->dim != 2) return fc;
   const Grid g0 = grid_of(h, 0), g1 = grid_of(h, 1);
   fc.ec = (const TU*)h->lv[1].u;
-  fc.dim = h->dim;
   fc.mf = g0.m;
   fc.mc = g1.m;
   fc.npc = g1.np;

@@ -328,7 +328,8 @@ cudaError_t launch_fevar3_objective_grad(Launch& L, int m, int n, double h, doub
                                          double* gg);
 
 // forward scaled time FFT: v (FP64 [2][n][ms]) -> spectral planes [2*nfreq][ms]
-// dpow[j] = eps^{j/n}, dinv[j] = eps^{-j/n}, tw[k] = exp(-2 pi i k/n) for k = 0..n-1
+// (twice the spectra: see k_tfft.cu)
+// dpow[j] = eps^{j/n}, dinv[j] = eps^{-j/n} / (2n), tw[k] = exp(-2 pi i k/n) for k = 0..n-1
 // With jdev != nullptr the input is v + (*jdev) * vstride (device-resident Arnoldi index).
 // input v: FP64 basis vectors, or (Tc = float) their FP32 rounding
 template <typename Tc, typename Tin = double>
@@ -338,13 +339,13 @@ cudaError_t launch_tfft_forward(Launch& L, int64_t ms, int n, const Tin* v, cons
 // inverse scaled time FFT + butterfly: spectral planes (stored as TU) -> w (Tout [2][n][ms])
 // With jdev != nullptr the output is w + (*jdev) * wstride.
 // Last step of the multigrid up leg, done while the inverse time transform loads
-// the finest level: u_f + P e_c, P the (bi/tri)linear prolongation from the next
+// the finest level of a 2D grid: u_f + P e_c, P the bilinear prolongation from the next
 // coarser level (mc = (mf - 1) / 2 points per axis, zero outside).  ec == nullptr:
 // the planes are used as they are.
 template <typename TU>
 struct FineCorrection {
   const TU* ec = nullptr;
-  int dim = 0, mf = 0, mc = 0;
+  int mf = 0, mc = 0;  // 2D grids
   int64_t npc = 0;
 };
 

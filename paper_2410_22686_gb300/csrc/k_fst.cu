@@ -52,14 +52,14 @@ __device__ __forceinline__ int xidx(int k2, int j1, int c) {
 // once every thread has read `src` (behind two barriers), between the first
 // exchange and the second register FFT: the persistent kernel refills `src` with
 // the next tile there.
-template <typename Tc, int N1, int N2, typename AfterRead>
+template <typename Tc, int N1, int N2, int NT, typename AfterRead>
 __device__ __forceinline__ void dst_tile(typename Cx<Tc>::t* sm, const typename Cx<Tc>::t* src,
                                          const typename Cx<Tc>::t* __restrict__ tw, int m, Tc half_scale, int r,
                                          int c, AfterRead&& after_read) {
   typedef typename Cx<Tc>::t C;
   constexpr int L = N1 * N2;
   constexpr int N = L / 2;
-  constexpr int COLS = 256 / N1;
+  constexpr int COLS = NT / N1;
   // (A) rows j = r + N1 j2 of the odd extension, N2-point DFT over j2
   C x[N2];
 #pragma unroll
@@ -75,7 +75,7 @@ __device__ __forceinline__ void dst_tile(typename Cx<Tc>::t* sm, const typename 
     x[j2] = v;
   }
   __syncthreads();  // every read of the tile is done before the exchange overwrites it
-  reg_fft<N2, false>(x, tw, N1);
+  dft_regs<N2, false>(x);
 #pragma unroll
   for (int k2 = 0; k2 < N2; ++k2) {
     const C y = (k2 == 0 || r == 0) ? x[k2] : cmul(tw[r * k2], x[k2]);
@@ -99,7 +99,7 @@ __device__ __forceinline__ void dst_tile(typename Cx<Tc>::t* sm, const typename 
 #pragma unroll
     for (int a = 0; a < H; ++a) y[a] = sm[xidx<N1, COLS>(k2, 2 * a + b, c)];
     __syncthreads();
-    reg_fft<H, false>(y, tw, 2 * N2);
+    dft_regs<H, false>(y);
 #pragma unroll
     for (int q = 0; q < H; ++q) {
       C v = y[q];
@@ -125,7 +125,7 @@ __device__ __forceinline__ void dst_tile(typename Cx<Tc>::t* sm, const typename 
     }
     __syncthreads();
     if (r < N2) {
-      reg_fft<N1, false>(y, tw, N2);
+      dft_regs<N1, false>(y);
 #pragma unroll
       for (int k1 = 0; k1 < N1; ++k1) put(r + N2 * k1, y[k1]);
     }
@@ -138,13 +138,13 @@ __device__ __forceinline__ void dst_tile(typename Cx<Tc>::t* sm, const typename 
 // tw[2q] and sin(pi j / N) = -Im tw[j].  `scale` = sqrt(2/N).  Same contract as
 // dst_tile: ends with a barrier; after_read() runs behind two barriers after every
 // read of `src`, when no transform values are held in registers.
-template <typename Tc, int N1, int N2, typename AfterRead>
+template <typename Tc, int N1, int N2, int NT, typename AfterRead>
 __device__ __forceinline__ void dsth_tile(typename Cx<Tc>::t* sm, const typename Cx<Tc>::t* src,
                                           const typename Cx<Tc>::t* __restrict__ tw, int m, Tc scale, int r, int c,
                                           AfterRead&& after_read) {
   typedef typename Cx<Tc>::t C;
   constexpr int N = N1 * N2;
-  constexpr int COLS = 256 / N1;
+  constexpr int COLS = NT / N1;
   constexpr int Q = N / 2 / N1;  // odd outputs per thread row
   static_assert(Q >= 1, "N must be at least 2 N1");
   __shared__ C tot[N1 * COLS];  // chunk totals of the prefix sum
@@ -160,7 +160,7 @@ __device__ __forceinline__ void dsth_tile(typename Cx<Tc>::t* sm, const typename
     x[j2] = cmk<Tc>(sj * (a.x + b.x) + h * (a.x - b.x), sj * (a.y + b.y) + h * (a.y - b.y));
   }
   __syncthreads();  // every read of the tile is done before the exchange overwrites it
-  reg_fft<N2, false>(x, tw, 2 * N1);
+  dft_regs<N2, false>(x);
 #pragma unroll
   for (int k2 = 0; k2 < N2; ++k2) {
     const C y = (k2 == 0 || r == 0) ? x[k2] : cmul(tw[2 * r * k2], x[k2]);
@@ -177,7 +177,7 @@ __device__ __forceinline__ void dsth_tile(typename Cx<Tc>::t* sm, const typename
     }
     __syncthreads();
     if (r < N2) {
-      reg_fft<N1, false>(y, tw, 2 * N2);
+      dft_regs<N1, false>(y);
 #pragma unroll
       for (int k1 = 0; k1 < N1; ++k1) sm[(r + N2 * k1) * COLS + c] = y[k1];
     }
@@ -215,14 +215,14 @@ __device__ __forceinline__ void dsth_tile(typename Cx<Tc>::t* sm, const typename
 // Lines: plane p = line / (np / m); inside the plane, a line along `axis` starts at
 // outer * m * lstride + inner with lstride = m^axis, inner < lstride.
 // one line-tile DST of the kind HALF selects (dsth_tile or dst_tile)
-template <typename Tc, int N1, int N2, bool HALF, typename AfterRead>
+template <typename Tc, int N1, int N2, bool HALF, int NT, typename AfterRead>
 __device__ __forceinline__ void dst_any(typename Cx<Tc>::t* sm, const typename Cx<Tc>::t* src,
                                         const typename Cx<Tc>::t* __restrict__ tw, int m, Tc scale, int r, int c,
                                         AfterRead&& after_read) {
   if constexpr (HALF)
-    dsth_tile<Tc, N1, N2>(sm, src, tw, m, scale, r, c, after_read);
+    dsth_tile<Tc, N1, N2, NT>(sm, src, tw, m, scale, r, c, after_read);
   else
-    dst_tile<Tc, N1, N2>(sm, src, tw, m, scale, r, c, after_read);
+    dst_tile<Tc, N1, N2, NT>(sm, src, tw, m, scale, r, c, after_read);
 }
 
 // CTAs per SM the kernels are compiled for (registers per thread = 65536 / (256 x it))
@@ -232,14 +232,14 @@ constexpr int fst_min_blocks() {
   return (NP <= 256 && !STREAM) ? 2 : 1;
 }
 
-template <typename Tc, int N1, int N2, bool DIVIDE, bool HALF>
-__global__ void __launch_bounds__(256, fst_min_blocks<Tc, N1 * N2, false>()) fst4_kernel(const typename Cx<Tc>::t* in, typename Cx<Tc>::t* out,
+template <typename Tc, int N1, int N2, bool DIVIDE, bool HALF, int NT>
+__global__ void __launch_bounds__(NT, fst_min_blocks<Tc, N1 * N2, false>() * (256 / NT)) fst4_kernel(const typename Cx<Tc>::t* in, typename Cx<Tc>::t* out,
                                                    const typename Cx<Tc>::t* __restrict__ tw, int m, int64_t np,
                                                    int64_t lstride, int64_t nlines, Tc half_scale,
                                                    const Tc* __restrict__ lamK, const Tc* __restrict__ rmass,
                                                    const typename Cx<Tc>::t* __restrict__ sigma) {
   typedef typename Cx<Tc>::t C;
-  constexpr int COLS = 256 / N1;
+  constexpr int COLS = NT / N1;
   extern __shared__ __align__(16) unsigned char fst_smem[];
   C* sm = reinterpret_cast<C*>(fst_smem);
   __shared__ int64_t lbase[COLS];  // offset of each line's first value (plane included)
@@ -261,15 +261,15 @@ __global__ void __launch_bounds__(256, fst_min_blocks<Tc, N1 * N2, false>()) fst
   }
   __syncthreads();
   const int tot = COLS * m;
-  for (int e = tid; e < tot; e += 256) {
+  for (int e = tid; e < tot; e += NT) {
     const int j = e / COLS, c = e - j * COLS;
     sm[e] = lplane[c] >= 0 ? in[lbase[c] + (int64_t)j * lstride] : czero<Tc>();
   }
   __syncthreads();
   const int r = tid / COLS, c = tid - (tid / COLS) * COLS;
-  dst_any<Tc, N1, N2, HALF>(sm, sm, tw, m, half_scale, r, c, [] {});
+  dst_any<Tc, N1, N2, HALF, NT>(sm, sm, tw, m, half_scale, r, c, [] {});
   if (DIVIDE) {
-    for (int e = tid; e < tot; e += 256) {
+    for (int e = tid; e < tot; e += NT) {
       const int j = e / COLS, cc = e - j * COLS;
       const int p = lplane[cc];
       if (p < 0) continue;
@@ -279,9 +279,9 @@ __global__ void __launch_bounds__(256, fst_min_blocks<Tc, N1 * N2, false>()) fst
       sm[e] = cmul(v, inv_diag<Tc>(sigma[p], lamK[s]));
     }
     __syncthreads();
-    dst_any<Tc, N1, N2, HALF>(sm, sm, tw, m, half_scale, r, c, [] {});
+    dst_any<Tc, N1, N2, HALF, NT>(sm, sm, tw, m, half_scale, r, c, [] {});
   }
-  for (int e = tid; e < tot; e += 256) {
+  for (int e = tid; e < tot; e += NT) {
     const int j = e / COLS, cc = e - j * COLS;
     if (lplane[cc] >= 0) out[lbase[cc] + (int64_t)j * lstride] = sm[e];
   }
@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(256, fst_min_blocks<Tc, N1 * N2, true>()) fst4
     cp_async_wait<0>();
     __syncthreads();  // the stage holds this tile; the previous tile's stores are done
     if (next < ntiles) bases(next, slot ^ 1);
-    dst_any<Tc, N1, N2, HALF>(sm, stage, tw, m, half_scale, r, c, [&] {
+    dst_any<Tc, N1, N2, HALF, 256>(sm, stage, tw, m, half_scale, r, c, [&] {
       if (next < ntiles) issue(slot ^ 1);
     });
     if (DIVIDE) {
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(256, fst_min_blocks<Tc, N1 * N2, true>()) fst4
         sm[e] = cmul(v, inv_diag<Tc>(sigma[p], lamK[s]));
       }
       __syncthreads();
-      dst_any<Tc, N1, N2, HALF>(sm, sm, tw, m, half_scale, r, c, [] {});
+      dst_any<Tc, N1, N2, HALF, 256>(sm, sm, tw, m, half_scale, r, c, [] {});
     }
     for (int e = tid; e < tot; e += 256) {
       const int j = e / COLS, cc = e - j * COLS;
@@ -384,17 +384,29 @@ cudaError_t fst4s(Launch& L, const Grid& g, int64_t lstride, int64_t nlines, Tc 
   return cudaGetLastError();
 }
 
+template <typename Tc, int N1, int N2, bool HALF, int NT>
+cudaError_t fst4_nt(Launch& L, const Grid& g, bool divide, int64_t lstride, int64_t nlines, Tc hs,
+                    const typename Cx<Tc>::t* tw, const Tc* lamK, const Tc* rmass, const typename Cx<Tc>::t* sigma,
+                    const typename Cx<Tc>::t* in, typename Cx<Tc>::t* out) {
+  constexpr int COLS = NT / N1;
+  const size_t smem = (size_t)(N1 + 1) * N2 * COLS * sizeof(typename Cx<Tc>::t);
+  const unsigned blocks = (unsigned)((nlines + COLS - 1) / COLS);
+  auto kern = divide ? fst4_kernel<Tc, N1, N2, true, HALF, NT> : fst4_kernel<Tc, N1, N2, false, HALF, NT>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kern<<<blocks, NT, smem, L.stream>>>(in, out, tw, g.m, g.np, lstride, nlines, hs, lamK, rmass, sigma);
+  return cudaGetLastError();
+}
+
 // HALF: N1 N2 = m + 1 (half-length DST); otherwise N1 N2 = 2(m + 1) (odd extension)
 template <typename Tc, int N1, int N2, bool HALF>
 cudaError_t fst4(Launch& L, const Grid& g, int planes, int axis, bool divide, const typename Cx<Tc>::t* tw,
                  const Tc* lamK, const Tc* rmass, const typename Cx<Tc>::t* sigma, const typename Cx<Tc>::t* in,
                  typename Cx<Tc>::t* out, bool stream) {
   constexpr int COLS = 256 / N1;
-  const size_t smem = (size_t)(N1 + 1) * N2 * COLS * sizeof(typename Cx<Tc>::t);
   int64_t lstride = 1;
   for (int a = 0; a < axis; ++a) lstride *= g.m;
   const int64_t nlines = (int64_t)planes * (g.np / g.m);
-  const unsigned blocks = (unsigned)((nlines + COLS - 1) / COLS);
   const double s2n = std::sqrt(2.0 / (g.m + 1));
   const Tc hs = (Tc)(HALF ? s2n : 0.5 * s2n);
   if constexpr (sizeof(Tc) == 4 || N1 * N2 <= 256) {  // FP64 at 512 points has no registers to spare
@@ -403,19 +415,13 @@ cudaError_t fst4(Launch& L, const Grid& g, int planes, int axis, bool divide, co
                     : fst4s<Tc, N1, N2, false, HALF>(L, g, lstride, nlines, hs, tw, nullptr, nullptr, nullptr, in,
                                                      out);
   }
-  cudaError_t e;
-  if (divide) {
-    auto kern = fst4_kernel<Tc, N1, N2, true, HALF>;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<blocks, 256, smem, L.stream>>>(in, out, tw, g.m, g.np, lstride, nlines, hs, lamK, rmass, sigma);
-  } else {
-    auto kern = fst4_kernel<Tc, N1, N2, false, HALF>;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<blocks, 256, smem, L.stream>>>(in, out, tw, g.m, g.np, lstride, nlines, hs, nullptr, nullptr, nullptr);
-  }
-  return cudaGetLastError();
+  // a quarter of the lines a CTA where 256 threads would leave fewer than two CTAs an SM
+  // (31^2 x 34 planes, FP64: 33 CTAs against 132, axis pass 15.2 -> 11.0 us,
+  // fused pass 29.2 -> 22.4, fewer operations included)
+  if constexpr (HALF && N1 >= 4 && N1 <= 16)
+    if ((nlines + COLS - 1) / COLS < 2 * num_sms())
+      return fst4_nt<Tc, N1, N2, HALF, 64>(L, g, divide, lstride, nlines, hs, tw, lamK, rmass, sigma, in, out);
+  return fst4_nt<Tc, N1, N2, HALF, 256>(L, g, divide, lstride, nlines, hs, tw, lamK, rmass, sigma, in, out);
 }
 
 }  // namespace

@@ -193,16 +193,15 @@ __global__ void __launch_bounds__(kCzThreads, 2) tchirp_forward_kernel(const Tin
   __syncthreads();
   cz_transform<Tc>(t, cz.logM, n, cz.chirp(), cz.filter(n));
   const int nf = n / 2 + 1;
-  const Tc hf = Tc(0.5);
   for (int e = threadIdx.x; e < nf << lc; e += kCzThreads) {
     const int k = e >> lc, c = e & ((1 << lc) - 1);
     const int64_t s = s0 + c;
     if (s >= ms) continue;
     const C Z = t.sm[(k << lc) + c];
     const C W = t.sm[((k == 0 ? 0 : n - k) << lc) + c];
-    // hat v2[k] = (Z[k] - conj Z[n-k]) / (2i);  hat v1[k] = (Z[k] + conj Z[n-k]) / 2
-    spec[(int64_t)(2 * k) * ms + s] = cmk<Tc>((Z.y + W.y) * hf, (W.x - Z.x) * hf);
-    spec[(int64_t)(2 * k + 1) * ms + s] = cmk<Tc>((Z.x + W.x) * hf, (Z.y - W.y) * hf);
+    // 2 hat v2[k] = -i (Z[k] - conj Z[n-k]);  2 hat v1[k] = Z[k] + conj Z[n-k] (as k_tfft.cu)
+    spec[(int64_t)(2 * k) * ms + s] = cmk<Tc>(Z.y + W.y, W.x - Z.x);
+    spec[(int64_t)(2 * k + 1) * ms + s] = cmk<Tc>(Z.x + W.x, Z.y - W.y);
   }
 }
 
@@ -228,8 +227,8 @@ __global__ void __launch_bounds__(kCzThreads, 2) tchirp_inverse_kernel(const TU*
       if (fc.ec) {
         Parents<Tc, TU> par;
         par.init(fc, s);
-        sa = sa + par.at(fc, 2 * k);
-        sb = sb + par.at(fc, 2 * k + 1);
+        sa = par.corrected(sa, fc, 2 * k);
+        sb = par.corrected(sb, fc, 2 * k + 1);
       }
     }
     // Y[k] = hat w1[k] + i hat w2[k], Y[n-k] = conj(hat w1[k]) + i conj(hat w2[k]), exchanged
@@ -238,7 +237,6 @@ __global__ void __launch_bounds__(kCzThreads, 2) tchirp_inverse_kernel(const TU*
   }
   __syncthreads();
   cz_transform<Tc>(t, cz.logM, n, cz.chirp(), cz.filter(n));
-  const Tc inv_n = Tc(1) / Tc(n);
   Tout* w1 = w;
   Tout* w2 = w + (int64_t)n * ms;
   for (int e = threadIdx.x; e < n << lc; e += kCzThreads) {
@@ -246,8 +244,8 @@ __global__ void __launch_bounds__(kCzThreads, 2) tchirp_inverse_kernel(const TU*
     const int64_t s = s0 + c;
     if (s >= ms) continue;
     const int jr = n - 1 - j;
-    const Tc wt1 = dinv[jr] * (t.sm[(jr << lc) + c].y * inv_n);  // J D^{-1} ifft(hat w1)
-    const Tc wt2 = dinv[j] * (t.sm[(j << lc) + c].x * inv_n);    // D^{-1} ifft(hat w2)
+    const Tc wt1 = dinv[jr] * t.sm[(jr << lc) + c].y;  // J D^{-1} ifft(hat w1)
+    const Tc wt2 = dinv[j] * t.sm[(j << lc) + c].x;    // D^{-1} ifft(hat w2)
     w1[(int64_t)j * ms + s] = cvt<Tout>(wt1 - wt2);  // step 4: [[I, -I], [I, I]]
     w2[(int64_t)j * ms + s] = cvt<Tout>(wt1 + wt2);
   }

@@ -15,39 +15,6 @@ __device__ __forceinline__ constexpr int brev_ct(int i) {
   return r;
 }
 
-// in-place R-point DFT of registers x (DIT, radix 2); twiddles exp(-+2 pi i q/R)
-// are tw[q * tstride] from the full-circle table of length n = R * tstride
-template <int R, bool INV, typename C>
-__device__ __forceinline__ void reg_fft(C (&x)[R], const C* __restrict__ tw, int tstride) {
-#pragma unroll
-  for (int i = 0; i < R; ++i) {
-    const int j = brev_ct<R>(i);
-    if (j > i) {
-      const C t = x[i];
-      x[i] = x[j];
-      x[j] = t;
-    }
-  }
-#pragma unroll
-  for (int half = 1; half < R; half <<= 1) {
-#pragma unroll
-    for (int g = 0; g < R; g += 2 * half) {
-#pragma unroll
-      for (int p = 0; p < half; ++p) {
-        const C a = x[g + p];
-        C b = x[g + p + half];
-        if (p != 0) {
-          C w = tw[p * (R / (2 * half)) * tstride];
-          if (INV) w.y = -w.y;
-          b = cmul(w, b);
-        }
-        x[g + p] = a + b;
-        x[g + p + half] = a - b;
-      }
-    }
-  }
-}
-
 // cos(2 pi q / 32) for q = 0..8
 template <typename T>
 __device__ __forceinline__ constexpr T cos32(int q) {
@@ -64,11 +31,14 @@ __device__ __forceinline__ constexpr T cos32(int q) {
   }
 }
 
-// In-place R-point DFT of registers (R <= 32), the twiddles compile-time constants.  A
-// butterfly with a twiddle takes six fused multiply-adds (a + w b in four, and a - w b as
-// 2 a - (a + w b)) where a product and two sums take eight; quarter turns cost the sums
-// alone.  16 points: 148 operations instead of 196.  HALF_IN: inputs R/2.. are zero;
-// HALF_OUT: only outputs 0..R/2-1 are wanted.
+// In-place R-point DFT of registers (R <= 32), the twiddles compile-time constants, quarter
+// turns costing their two sums alone.  In FP64, whose unit bounds the transforms, a butterfly
+// with another twiddle takes six fused multiply-adds (a + w b in four, a - w b as
+// 2 a - (a + w b)) where a product and two sums take eight: 148 operations for 16 points
+// instead of 196 (preconditioner apply in FP64, 31^2: n = 256 2.24e-15 off against 2.26e-15
+// before).  In FP32, bound elsewhere, the sums follow the product: the fused form's error is
+// 1-2% larger there.  HALF_IN: inputs R/2.. are zero; HALF_OUT: only outputs 0..R/2-1 are
+// wanted.
 template <int R, bool INV, bool HALF_IN = false, bool HALF_OUT = false, typename C>
 __device__ __forceinline__ void dft_regs(C (&x)[R]) {
   typedef decltype(C().x) T;
@@ -106,12 +76,20 @@ __device__ __forceinline__ void dft_regs(C (&x)[R]) {
           const T ws = q <= 8 ? cos32<T>(8 - q) : cos32<T>(q - 8);
           const T wi = INV ? ws : -ws;
           C t;
-          t.x = fma(-wi, b.y, fma(wr, b.x, a.x));
-          t.y = fma(wi, b.x, fma(wr, b.y, a.y));
-          x[g + p] = t;
-          if (!last) {
-            x[g + p + half].x = fma(T(2), a.x, -t.x);
-            x[g + p + half].y = fma(T(2), a.y, -t.y);
+          if (sizeof(T) == 8) {
+            t.x = fma(-wi, b.y, fma(wr, b.x, a.x));
+            t.y = fma(wi, b.x, fma(wr, b.y, a.y));
+            x[g + p] = t;
+            if (!last) {
+              x[g + p + half].x = fma(T(2), a.x, -t.x);
+              x[g + p + half].y = fma(T(2), a.y, -t.y);
+            }
+          } else {
+            t.x = wr;
+            t.y = wi;
+            t = cmul(t, b);
+            x[g + p] = a + t;
+            if (!last) x[g + p + half] = a - t;
           }
         }
       }
