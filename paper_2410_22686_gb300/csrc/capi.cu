@@ -1175,40 +1175,24 @@ static cudaError_t spatial_solve(pc_handle* h, Launch& L, int nplanes = 0,
   const C* sig = sig_override ? sig_override : Tables<Tc>::sig(h);
   cudaError_t e;
   if constexpr (std::is_same<TU, C>::value) {
-    if (h->spatial == PC_SPATIAL_FST && Tables<Tc>::fst_tw(h) && fst_fast_supported<Tc>(h->m1)) {
-      // fast transforms: forward along x1 (.. x_{d-1}), the last axis fused with the
-      // divide, inverse back down to x1
+    if (h->spatial == PC_SPATIAL_FST) {
+      // forward along x1 (.. x_{d-1}), the last axis fused with the divide, inverse back down
+      // to x1: register FFTs where m + 1 is a power of two they take, else matrix products
       const Grid g = grid_of(h, 0);
-      const C* tw = Tables<Tc>::fst_tw(h);
+      const bool fast = Tables<Tc>::fst_tw(h) && fst_fast_supported<Tc>(h->m1);
+      auto axis = [&](int ax, bool divide, const C* in, C* out) {
+        const Tc *lam = divide ? Tables<Tc>::lamK(h) : nullptr, *rm = divide ? Tables<Tc>::rmass(h) : nullptr;
+        const C* sg = divide ? sig : nullptr;
+        return fast ? launch_fst_fast<Tc>(L, g, P, ax, divide, Tables<Tc>::fst_tw(h), lam, rm, sg, in, out)
+                    : launch_dst_dense<Tc>(L, g, P, ax, divide, Tables<Tc>::S(h), lam, rm, sg, in, out);
+      };
       C* tmp = (C*)h->fst_tmp;
       const int last = h->dim - 1;
       for (int ax = 0; ax < last; ++ax)
-        if ((e = launch_fst_fast<Tc>(L, g, P, ax, false, tw, nullptr, nullptr, nullptr, ax == 0 ? (const C*)h->lv[0].r : tmp,
-                                     tmp)) != cudaSuccess)
-          return e;
-      if ((e = launch_fst_fast<Tc>(L, g, P, last, true, tw, Tables<Tc>::lamK(h), Tables<Tc>::rmass(h), sig, tmp,
-                                   last == 0 ? (C*)h->lv[0].u : tmp)) != cudaSuccess)
-        return e;
+        if ((e = axis(ax, false, ax == 0 ? (const C*)h->lv[0].r : tmp, tmp)) != cudaSuccess) return e;
+      if ((e = axis(last, true, tmp, tmp)) != cudaSuccess) return e;
       for (int ax = last - 1; ax >= 0; --ax)
-        if ((e = launch_fst_fast<Tc>(L, g, P, ax, false, tw, nullptr, nullptr, nullptr, tmp,
-                                     ax == 0 ? (C*)h->lv[0].u : tmp)) != cudaSuccess)
-          return e;
-      return cudaSuccess;
-    }
-    if (h->spatial == PC_SPATIAL_FST) {
-      const Grid g = grid_of(h, 0);
-      C* bufs[2] = {(C*)h->lv[0].r, (C*)h->fst_tmp};
-      int cur = 0;
-      for (int ax = 0; ax < h->dim; ++ax) {
-        if ((e = launch_fst_axis<Tc>(L, g, P, ax, Tables<Tc>::S(h), bufs[cur], bufs[1 - cur])) != cudaSuccess) return e;
-        cur = 1 - cur;
-      }
-      if ((e = launch_fst_divide<Tc>(L, g, P, Tables<Tc>::lamK(h), Tables<Tc>::rmass(h), sig, bufs[cur])) != cudaSuccess) return e;
-      for (int ax = h->dim - 1; ax >= 0; --ax) {
-        C* dst = ax == 0 ? (C*)h->lv[0].u : bufs[1 - cur];
-        if ((e = launch_fst_axis<Tc>(L, g, P, ax, Tables<Tc>::S(h), bufs[cur], dst)) != cudaSuccess) return e;
-        cur = 1 - cur;
-      }
+        if ((e = axis(ax, false, tmp, ax == 0 ? (C*)h->lv[0].u : tmp)) != cudaSuccess) return e;
       return cudaSuccess;
     }
   }

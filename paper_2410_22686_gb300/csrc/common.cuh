@@ -376,14 +376,13 @@ template <typename Tc, typename TU, typename Tout>
 cudaError_t launch_tchirp_inverse(Launch& L, int64_t ms, int n, const TU* spec, const Tc* dinv, ChirpZ<Tc> cz, Tout* w,
                                   FineCorrection<TU> fc);
 
-// FST: one DST-I along `axis` of every plane (out = S in), and the spectral divide
-// buf *= rmass / (sigma + lamK) (rmass == nullptr: 1)
+// Sine transforms of any m (k_dst.cu): out = S in along `axis` (S the orthonormal DST-I), or
+// with `divide` out = S diag(rmass / (sigma_p + lamK)) S in (rmass == nullptr: 1).  in may
+// equal out.
 template <typename Tc>
-cudaError_t launch_fst_axis(Launch& L, const Grid& g, int planes, int axis, const Tc* S,
-                            const typename Cx<Tc>::t* in, typename Cx<Tc>::t* out);
-template <typename Tc>
-cudaError_t launch_fst_divide(Launch& L, const Grid& g, int planes, const Tc* lamK, const Tc* rmass,
-                              const typename Cx<Tc>::t* sigma, typename Cx<Tc>::t* buf);
+cudaError_t launch_dst_dense(Launch& L, const Grid& g, int planes, int axis, bool divide, const Tc* S, const Tc* lamK,
+                             const Tc* rmass, const typename Cx<Tc>::t* sigma, const typename Cx<Tc>::t* in,
+                             typename Cx<Tc>::t* out);
 // Fast sine transforms (k_fst.cu) for m + 1 a power of two, 2(m+1) <= 1024 (FP32) /
 // 512 (FP64): out = S in along `axis` (S the orthonormal DST-I), or with `divide`
 // out = S diag(rmass / (sigma_p + lamK)) S in along the last axis.  tw: the

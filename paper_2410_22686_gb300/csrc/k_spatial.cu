@@ -1,9 +1,9 @@
 // Step 2 of the four-step apply of P_eps^{-1} (Section 2.1): for every
 // spectral plane p (frequency k = p/2, shift sigma_p = lambda_k + alpha) solve
 //     (sigma_p I + tau K) u_p = r_p
-// either exactly by sine transforms (constant a, Example 1) or approximately
-// by one V(1,0) multigrid cycle (variable a, Example 2: Gauss-Seidel
-// pre-smoother, no post-smoother).  The multigrid reading: one red-black
+// approximately by one V(1,0) multigrid cycle (variable a, Example 2: Gauss-Seidel
+// pre-smoother, no post-smoother; the exact sine-transform solves of a constant a are in
+// k_fst.cu and k_dst.cu).  The multigrid reading: one red-black
 // Gauss-Seidel sweep from zero (red = even sum of 1-based indices, first),
 // full-weighting restriction, (bi/tri)linear prolongation, rediscretised
 // coarse operators with the nodal coefficient injected, the same shift on
@@ -45,43 +45,6 @@ __device__ __forceinline__ Coord coord_of(int64_t s, int m, int dim) {
     c.i3 = (int)(r / m);
   }
   return c;
-}
-
-// ------------------------------------------------------------------- FST
-template <typename Tc>
-__global__ void fst_axis_kernel(const typename Cx<Tc>::t* __restrict__ in, typename Cx<Tc>::t* __restrict__ out,
-                                const Tc* __restrict__ S, int m, int dim, int axis, int64_t np, int planes) {
-  typedef typename Cx<Tc>::t C;
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= np * planes) return;
-  const int64_t p = e / np;
-  const int64_t s = e - p * np;
-  const Coord c = coord_of(s, m, dim);
-  const int i = axis == 0 ? c.i1 : (axis == 1 ? c.i2 : c.i3);
-  int64_t stride = 1;
-  for (int a = 0; a < axis; ++a) stride *= m;
-  const C* src = in + p * np + (s - (int64_t)i * stride);
-  Tc ar = 0, ai = 0;
-  for (int j = 0; j < m; ++j) {
-    const Tc sij = S[i * m + j];
-    const C v = src[(int64_t)j * stride];
-    ar = fma(sij, v.x, ar);
-    ai = fma(sij, v.y, ai);
-  }
-  out[e] = cmk<Tc>(ar, ai);
-}
-
-template <typename Tc>
-__global__ void fst_divide_kernel(typename Cx<Tc>::t* __restrict__ buf, const Tc* __restrict__ lamK,
-                                  const Tc* __restrict__ rmass, const typename Cx<Tc>::t* __restrict__ sigma,
-                                  int64_t np, int planes) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= np * planes) return;
-  const int64_t p = e / np;
-  const int64_t s = e - p * np;
-  typename Cx<Tc>::t v = buf[e];
-  if (rmass) v = cscale(v, rmass[s]);  // finite elements: 1 / eigenvalue of M
-  buf[e] = cmul(v, inv_diag<Tc>(sigma[p], lamK[s]));
 }
 
 // ------------------------------------------------------------------- multigrid
@@ -564,27 +527,6 @@ int plane_chunk(const Launch& L) {
 
 }  // namespace
 
-template <typename Tc>
-cudaError_t launch_fst_axis(Launch& L, const Grid& g, int planes, int axis, const Tc* S,
-                            const typename Cx<Tc>::t* in, typename Cx<Tc>::t* out) {
-  const int64_t tot = g.np * planes;
-  const double cs = sizeof(typename Cx<Tc>::t);
-  L.begin(KC_FST_AXIS);
-  fst_axis_kernel<Tc><<<(unsigned)((tot + 255) / 256), 256, 0, L.stream>>>(in, out, S, g.m, g.dim, axis, g.np, planes);
-  return L.end(KC_FST_AXIS, 2.0 * tot * cs, 4.0 * tot * g.m);
-}
-
-template <typename Tc>
-cudaError_t launch_fst_divide(Launch& L, const Grid& g, int planes, const Tc* lamK, const Tc* rmass,
-                              const typename Cx<Tc>::t* sigma,
-                              typename Cx<Tc>::t* buf) {
-  const int64_t tot = g.np * planes;
-  const double cs = sizeof(typename Cx<Tc>::t);
-  L.begin(KC_FST_DIVIDE);
-  fst_divide_kernel<Tc><<<(unsigned)((tot + 255) / 256), 256, 0, L.stream>>>(buf, lamK, rmass, sigma, g.np, planes);
-  return L.end(KC_FST_DIVIDE, 2.0 * tot * cs, 12.0 * tot);
-}
-
 template <typename Tc, typename TU>
 cudaError_t launch_mg_smooth(Launch& L, const Grid& g, int planes, const Stencil<Tc>& st,
                              const typename Cx<Tc>::t* sigma, const typename Cx<Tc>::t* r, TU* u) {
@@ -695,10 +637,6 @@ cudaError_t launch_mg_coarsest(Launch& L, int planes, const Tc* diag, const type
   return L.end(KC_MG_COARSEST, 2.0 * planes * cs, 12.0 * planes);
 }
 
-#define PCOPT_INST_FST(Tc)                                                                                   \
-  template cudaError_t launch_fst_axis<Tc>(Launch&, const Grid&, int, int, const Tc*, const Cx<Tc>::t*,          \
-                                           Cx<Tc>::t*);                                                             \
-  template cudaError_t launch_fst_divide<Tc>(Launch&, const Grid&, int, const Tc*, const Tc*, const Cx<Tc>::t*, Cx<Tc>::t*);
 #define PCOPT_INST_MG(Tc, TU)                                                                                    \
   template cudaError_t launch_mg_smooth<Tc, TU>(Launch&, const Grid&, int, const Stencil<Tc>&, const Cx<Tc>::t*, \
                                                 const Cx<Tc>::t*, TU*);                                             \
@@ -710,12 +648,9 @@ cudaError_t launch_mg_coarsest(Launch& L, int planes, const Tc* diag, const type
   template cudaError_t launch_mg_prolong<Tc, TU>(Launch&, const Grid&, int, const TU*, TU*);                     \
   template cudaError_t launch_mg_coarsest<Tc, TU>(Launch&, int, const Tc*, const Cx<Tc>::t*, const Cx<Tc>::t*,   \
                                                   TU*);
-PCOPT_INST_FST(float)
-PCOPT_INST_FST(double)
 PCOPT_INST_MG(float, float2)
 PCOPT_INST_MG(double, double2)
 PCOPT_INST_MG(float, __nv_bfloat162)
-#undef PCOPT_INST_FST
 #undef PCOPT_INST_MG
 
 }  // namespace pcopt
