@@ -606,6 +606,7 @@ int num_sms();
 // time blocks per thread of a double-float product launched with `blocks` CTAs per chunk of
 // time, for at least per_sm CTAs an SM (k_matvec.cu); tuned > 0 overrides
 int time_chunk_filling(int64_t blocks, int n, int per_sm, int tuned);
+int time_chunk_balanced(int64_t blocks, int n);
 
 // record `msg` as the calling thread's last error (pc_last_error) and return `status`
 int set_error(int status, const std::string& msg);

@@ -14,6 +14,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "dfloat.cuh"
 
 namespace pcopt {
 
@@ -427,43 +428,23 @@ __global__ void __launch_bounds__(256) fevar_level_elements_kernel(const double*
 
 // ---------------------------------------------------------------------------
 // Element product of an FP32 vector (the inner product of flexible GMRES) in
-// double-float arithmetic: the nine K entries of a point are split once into FP32
-// (hi, lo) pairs; per time block and half, M u (integer weights on FP32 values, every
+// double-float arithmetic: the nine K entries of a point, times tau, are split once into
+// FP32 (hi, lo) pairs; per time block and half, M u (integer weights on FP32 values, every
 // term exact) and K u (exact products hi * u by FMA, lo * u rounded) are summed with
 // Knuth's TwoSum into (sum, error) pairs, widened on the integer pipes and combined
-// in FP64 (a few FP64 operations per output instead of ~45).  Relative error of a
-// sum: about 2^-44 of the sum of the magnitudes of its terms.
+// in FP64.  Relative error of a sum: about 2^-44 of the sum of the magnitudes of its terms.
+// Bound by the FP64 unit and the issue rate together: three FP64 operations an output, six
+// before K was kept times tau and the sums were widened with no FP64 addition (with the
+// chunks of time balanced over the SMs, 127^2 x 128: 76.9 -> 62.7 us, 255^2 x 256: 477 -> 371).
 // ---------------------------------------------------------------------------
 namespace {
-
-struct DF {
-  float hi, lo;
-};
-
-// (hi, lo) += x exactly (TwoSum; no contraction into FMA)
-__device__ __forceinline__ void df_add(DF& a, float x) {
-  const float s = __fadd_rn(a.hi, x);
-  const float bb = __fsub_rn(s, a.hi);
-  const float err = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bb)), __fsub_rn(x, bb));
-  a.hi = s;
-  a.lo = __fadd_rn(a.lo, err);
-}
-
-// (hi, lo) += (kh + kl) u
-__device__ __forceinline__ void df_add_prod(DF& a, float kh, float kl, float u) {
-  const float p = __fmul_rn(kh, u);
-  const float e = fmaf(kh, u, -p);
-  df_add(a, p);
-  a.lo = __fadd_rn(a.lo, fmaf(kl, u, e));
-}
-
-__device__ __forceinline__ double df_val(const DF& a) { return f32_to_f64(a.hi) + f32_to_f64(a.lo); }
 
 struct KSplit {
   float h[9], l[9];  // centre, e, w, n, s, ne, nw, se, sw
 };
 
-__device__ __forceinline__ void mk_apply_df(const float* __restrict__ u, const KSplit& k, int m, int i1, int i2,
+// mu36 = (M u)_s 36 / h^2, ku = tau (K u)_s (p: the exponent of k's scale)
+__device__ __forceinline__ void mk_apply_df(const float* __restrict__ u, const KSplit& k, int p, int m, int i1, int i2,
                                             double& mu36, double& ku) {
   const int s = i2 * m + i1;
   const bool w = i1 > 0, e = i1 < m - 1, so = i2 > 0, no = i2 < m - 1;
@@ -478,15 +459,15 @@ __device__ __forceinline__ void mk_apply_df(const float* __restrict__ u, const K
   DF ak{0.0f, 0.0f};
 #pragma unroll
   for (int q = 0; q < 9; ++q) df_add_prod(ak, k.h[q], k.l[q], v[q]);
-  mu36 = df_val(am);
-  ku = df_val(ak);
+  mu36 = df_to_f64(am, 0);
+  ku = df_to_f64(ak, p);
 }
 
 template <bool TRANSPOSE>
 __global__ void __launch_bounds__(256) fevar_matvec_df_kernel(const float* __restrict__ x, double* __restrict__ y,
                                                               const double* __restrict__ E, int m, int n, int tj,
-                                                              double h2, double alpha, double tau, size_t xstride,
-                                                              size_t ystride, const int* __restrict__ jdev) {
+                                                              double h2, double alpha, double tau, int p,
+                                                              size_t xstride, size_t ystride, const int* __restrict__ jdev) {
   const int64_t np = (int64_t)m * m;
   const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= np) return;
@@ -500,44 +481,44 @@ __global__ void __launch_bounds__(256) fevar_matvec_df_kernel(const float* __res
   KSplit k;
   {
     const KStencil<double> kd = k_stencil(E, m, i1, i2);
+    const double ts = scalbn(tau, p);
     const double kv[9] = {kd.c, kd.e, kd.w, kd.n, kd.s, kd.ne, kd.nw, kd.se, kd.sw};
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
-      k.h[q] = f64_to_f32(kv[q]);
-      k.l[q] = f64_to_f32(kv[q] - f32_to_f64(k.h[q]));
+      const double v = kv[q] * ts;
+      k.h[q] = f64_to_f32(v);
+      k.l[q] = f64_to_f32(v - f32_to_f64(k.h[q]));
     }
   }
-  const double mh = h2 / 36.0, sg = TRANSPOSE ? -1.0 : 1.0;
+  // M = mh S, S the integer sums; y1 = alpha mh S x1_j + sg mh (S x2_j - S x2_{j+1}) + sg tau K x2_j,
+  // y2 = alpha mh S x2_j - sg mh (S x1_j - S x1_{j-1}) - sg tau K x1_j
+  constexpr double sg = TRANSPOSE ? -1.0 : 1.0;
+  const double mh = sg * (h2 / 36.0), am = alpha * (h2 / 36.0);
   const float* x1 = x;
   const float* x2 = x + (int64_t)n * np;
   double* y1 = y;
   double* y2 = y + (int64_t)n * np;
-  double Mx1p = 0.0;
+  double s1p = 0.0;
   if (j0 > 0) {
-    double mu, ku;
-    mk_apply_df(x1 + (int64_t)(j0 - 1) * np, k, m, i1, i2, mu, ku);
-    Mx1p = mh * mu;
+    double ku;
+    mk_apply_df(x1 + (int64_t)(j0 - 1) * np, k, p, m, i1, i2, s1p, ku);
   }
-  double pMx1 = 0.0, pMx2 = 0.0, pKx2 = 0.0;
+  double y1p = 0.0;  // y1 of the block before, but for its S x2_{j+1}
   for (int j = j0; j < j1; ++j) {
-    double mu1, ku1, mu2, ku2;
-    mk_apply_df(x1 + (int64_t)j * np, k, m, i1, i2, mu1, ku1);
-    mk_apply_df(x2 + (int64_t)j * np, k, m, i1, i2, mu2, ku2);
-    const double Mx1 = mh * mu1, Mx2 = mh * mu2;
-    y2[(int64_t)j * np + s] = alpha * Mx2 - sg * (Mx1 - Mx1p + tau * ku1);
-    if (j > j0) y1[(int64_t)(j - 1) * np + s] = alpha * pMx1 + sg * (pMx2 - Mx2 + tau * pKx2);
-    Mx1p = Mx1;
-    pMx1 = Mx1;
-    pMx2 = Mx2;
-    pKx2 = ku2;
+    double s1, k1, s2, k2;
+    mk_apply_df(x1 + (int64_t)j * np, k, p, m, i1, i2, s1, k1);
+    mk_apply_df(x2 + (int64_t)j * np, k, p, m, i1, i2, s2, k2);
+    y2[(int64_t)j * np + s] = fma(am, s2, fma(-mh, s1, fma(mh, s1p, TRANSPOSE ? k1 : -k1)));
+    if (j > j0) y1[(int64_t)(j - 1) * np + s] = fma(-mh, s2, y1p);
+    y1p = fma(am, s1, fma(mh, s2, TRANSPOSE ? -k2 : k2));
+    s1p = s1;
   }
-  double Mx2n = 0.0;
+  double s2n = 0.0;
   if (j1 < n) {
-    double mu, ku;
-    mk_apply_df(x2 + (int64_t)j1 * np, k, m, i1, i2, mu, ku);
-    Mx2n = mh * mu;
+    double ku;
+    mk_apply_df(x2 + (int64_t)j1 * np, k, p, m, i1, i2, s2n, ku);
   }
-  y1[(int64_t)(j1 - 1) * np + s] = alpha * pMx1 + sg * (pMx2 - Mx2n + tau * pKx2);
+  y1[(int64_t)(j1 - 1) * np + s] = fma(-mh, s2n, y1p);
 }
 
 }  // namespace
@@ -559,16 +540,18 @@ template <typename Tin>
 cudaError_t launch_matvec_fevar(Launch& L, int m, int n, double h2, double alpha, double tau, const double* E,
                                 const Tin* x, double* y, bool transpose, size_t xstride, size_t ystride,
                                 const int* jdev) {
-  const int tj = n < 16 ? n : 16;
+  const int64_t blocks = ((int64_t)m * m + 255) / 256;
+  const int tj = std::is_same<Tin, float>::value ? time_chunk_balanced(blocks, n) : time_chunk_filling(blocks, n, 3, 0);
   const dim3 grid = grid2((int64_t)m * m, (n + tj - 1) / tj);
   const double tot = 2.0 * n * (double)m * m;
   L.begin(KC_MATVEC);
   if constexpr (std::is_same<Tin, float>::value) {
+    const int p = df_scale_exponent(tau);
     if (transpose)
-      fevar_matvec_df_kernel<true><<<grid, 256, 0, L.stream>>>(x, y, E, m, n, tj, h2, alpha, tau, xstride, ystride,
+      fevar_matvec_df_kernel<true><<<grid, 256, 0, L.stream>>>(x, y, E, m, n, tj, h2, alpha, tau, p, xstride, ystride,
                                                                jdev);
     else
-      fevar_matvec_df_kernel<false><<<grid, 256, 0, L.stream>>>(x, y, E, m, n, tj, h2, alpha, tau, xstride, ystride,
+      fevar_matvec_df_kernel<false><<<grid, 256, 0, L.stream>>>(x, y, E, m, n, tj, h2, alpha, tau, p, xstride, ystride,
                                                                 jdev);
     return L.end(KC_MATVEC, tot * (sizeof(Tin) + 8.0), tot * 160.0);
   }

@@ -279,6 +279,26 @@ int time_chunk_filling(int64_t blocks, int n, int per_sm, int tuned) {
   return tj < n ? tj : n;
 }
 
+// Time blocks per thread of the FP32-input element products with a nodal coefficient, `blocks`
+// CTAs a chunk of time.  Issue-bound, a few CTAs an SM: the SM with the most CTAs ends last, and a chunk's
+// start (K entries, two mass products) costs about one more time block, so the chunk is the
+// one of the least max-CTAs-an-SM * (blocks a chunk + 1): 31^3 x 64 takes 13 (5 chunks, 3.85
+// CTAs an SM) where 16 left 3.08.  (Their FP64 products fill the chip and no further: at
+// 31^3 x 64 they take 506 us at 16 blocks and 527 at 13.)
+int time_chunk_balanced(int64_t blocks, int n) {
+  const int64_t sms = num_sms();
+  int best = 1;
+  int64_t least = INT64_MAX;
+  for (int tj = std::min(n, 32); tj >= 1; --tj) {
+    const int64_t ctas = blocks * ((n + tj - 1) / tj), cost = (ctas + sms - 1) / sms * (tj + 1);
+    if (cost < least) {
+      least = cost;
+      best = tj;
+    }
+  }
+  return best;
+}
+
 cudaError_t launch_matvec_df(Launch& L, const Grid& g, int n, const float2* w, const float2* diag, float2 alpha,
                              const float* x, double* y, size_t xstride, size_t ystride, const int* jdev) {
   const int threads = 256;
