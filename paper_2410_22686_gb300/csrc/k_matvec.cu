@@ -11,6 +11,8 @@
 // neighbours come through L1/L2 (the rows above/below belong to blocks that
 // run concurrently on the same time chunk).  DRAM traffic is the minimum:
 // read x once, write y once.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace pcopt {
