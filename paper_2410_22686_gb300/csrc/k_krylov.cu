@@ -147,22 +147,26 @@ __global__ void __launch_bounds__(kThreads) multidot_kernel(const double* __rest
 }
 
 // Device-resident Arnoldi index: nv = *jdev + 1 vectors, w = wbase + (*jdev + 1) wstride;
-// the chunk [i0, i0 + 16) exits when it lies beyond nv, otherwise dispatches on its count.
-// The norm column is ld - 1.
-template <bool WITH_NORM, bool LP = false>
-__global__ void __launch_bounds__(kThreads) multidot_dyn_kernel(const double* __restrict__ V, size_t ldv, int i0,
+// blockIdx.y is the chunk of 16 vectors: it exits when it lies beyond nv, otherwise dispatches
+// on its count.  The first chunk also forms w . w if `norm` (column ld - 1).
+template <bool LP>
+__global__ void __launch_bounds__(kThreads) multidot_dyn_kernel(const double* __restrict__ V, size_t ldv,
                                                                 const double* __restrict__ wbase, size_t wstride,
                                                                 const int* __restrict__ jdev, size_t len,
-                                                                double* __restrict__ partial, int ld,
+                                                                double* __restrict__ partial, int ld, bool norm,
                                                                 const double* __restrict__ gate) {
   if (gated_off(gate)) return;
-  const int nv = *jdev + 1;
+  const int nv = *jdev + 1, i0 = (int)blockIdx.y * kChunk;
   if (i0 >= nv) return;
   const double* w = wbase + (size_t)nv * wstride;
   const int cnt = nv - i0 < kChunk ? nv - i0 : kChunk;
+  const bool with_norm = !LP && norm && i0 == 0;
   switch (cnt) {
 #define PCOPT_DYN(k) \
-  case k: multidot_body<k, WITH_NORM, LP>(V, ldv, i0, w, len, partial, ld - 1, ld); break;
+  case k: \
+    if (with_norm) multidot_body<k, !LP, LP>(V, ldv, i0, w, len, partial, ld - 1, ld); \
+    else multidot_body<k, false, LP>(V, ldv, i0, w, len, partial, ld - 1, ld); \
+    break;
     PCOPT_DYN(1) PCOPT_DYN(2) PCOPT_DYN(3) PCOPT_DYN(4) PCOPT_DYN(5) PCOPT_DYN(6) PCOPT_DYN(7) PCOPT_DYN(8)
     PCOPT_DYN(9) PCOPT_DYN(10) PCOPT_DYN(11) PCOPT_DYN(12) PCOPT_DYN(13) PCOPT_DYN(14) PCOPT_DYN(15) PCOPT_DYN(16)
 #undef PCOPT_DYN
@@ -553,10 +557,11 @@ __global__ void loop_start_kernel(int* jdev, int* kdev, const double* est, doubl
 // (a producer warp issues the bulk asynchronous copies of several stages ahead on
 // mbarriers); the selective second pass reads the hi planes directly.
 // ---------------------------------------------------------------------------
-constexpr int kTile = 512;             // elements per tile of the layout and per streamed stage (two per thread)
+constexpr int kTile = 256;             // elements per tile of the layout and per streamed stage (two per thread)
 constexpr int kGroup = 16;             // basis vectors per stage of the update
 constexpr int kBarBytes = 256;         // mbarriers (16 full, 16 empty) at the start of the dynamic shared memory
-constexpr size_t kStreamSmem = 220 * 1024;  // dynamic shared-memory budget of a streaming CTA
+constexpr int kStreamCtas = 2;         // streaming CTAs an SM
+constexpr size_t kStreamSmem = 103 * 1024;  // dynamic shared-memory budget of a streaming CTA
 
 __device__ __forceinline__ float neg_f(float x) { return -x; }
 
@@ -625,66 +630,93 @@ __host__ __device__ __forceinline__ void balanced_chunk(int nv, int c, int* i0, 
   *i0 = c * base + (c < rem ? c : rem);
 }
 
-// Producer/consumer stream of a CTA's items through S shared-memory stages.
-// The CTA has kThreads consumer threads (warps 0..7) and one producer warp (warp
-// 8).  Stage q has a "full" mbarrier (one arrival with the copies' byte count,
-// completed by the copy engine) and an "empty" one (one arrival per consumer
-// warp once it has read the stage).  The producer's lanes issue an item's copies
-// together: issue(k, stage, full, lane).  consume(k, stage) runs on every consumer
-// thread.  No CTA-wide barrier inside the stream.  Every wait is bounded; one that
-// runs out sets *err, ends that thread's loop, and the producer then drains the
-// copies it has in flight (bounded) before the CTA leaves.
-constexpr int kConsumerWarps = kThreads / 32;
-constexpr int kStreamThreads = kThreads + 32;
+// bytes of a stage of `cnt` vectors' tiles and w's, and the stages of `stride` bytes that fit
+// the streaming CTA's shared-memory budget
+__host__ __device__ __forceinline__ size_t stage_stride_of(int cnt) {
+  return (size_t)2 * cnt * kTile * 4 + (size_t)kTile * 8;  // a multiple of 128
+}
+__host__ __device__ __forceinline__ int stream_stages_for(size_t stride) {
+  const size_t s = (kStreamSmem - kBarBytes) / stride;
+  return (int)(s < 2 ? 2 : (s > 12 ? 12 : s));
+}
 
-template <typename Issue, typename Consume>
-__device__ __forceinline__ void stream_items(size_t nitems, int S, size_t stage_stride, Issue issue, Consume consume,
-                                             double* err) {
+// Producer/consumer stream of a CTA's items through S shared-memory stages.
+// The CTA has kTile / 2 consumer threads and one producer warp, its last.  Stage q has a
+// "full" mbarrier (one arrival with the copies' byte count, completed by the copy engine)
+// and an "empty" one (one arrival per consumer warp once it has read the stage).  The
+// producer's lanes issue an item's copies together: issue(m, stage, full, lane).
+// consume(m, stage) runs on every consumer thread.  No CTA-wide barrier inside the stream.
+// A kernel may stream several runs of items: both sides count them on from k, so the
+// barriers keep their phases and the producer starts on the next run while the consumers
+// finish the last.  Every wait is bounded; one that runs out sets *err, ends the thread's
+// part (false), and the producer then drains the copies it has in flight (bounded).
+constexpr int kConsumerWarps = kTile / 64;
+constexpr int kStreamThreads = kTile / 2 + 32;
+
+struct Stream {
+  uint64_t *full, *empty;
+  unsigned char* buf;
+  size_t stride;
+  int S;
+};
+
+__device__ __forceinline__ Stream stream_begin(int S, size_t stage_stride) {
   extern __shared__ __align__(128) unsigned char dsm[];
-  uint64_t* full = reinterpret_cast<uint64_t*>(dsm);
-  uint64_t* empty = full + 16;
-  unsigned char* buf = dsm + kBarBytes;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(dsm);
+  const Stream st{bars, bars + 16, dsm + kBarBytes, stage_stride, S};
   if (threadIdx.x == 0) {
     for (int q = 0; q < S; ++q) {
-      mbar_init(&full[q], 1);
-      mbar_init(&empty[q], kConsumerWarps);
+      mbar_init(&st.full[q], 1);
+      mbar_init(&st.empty[q], kConsumerWarps);
     }
     mbar_init_fence();
   }
   __syncthreads();
-  if (warp == kConsumerWarps) {  // producer
-    size_t k = 0;
-    bool ok = true;
-    for (; k < nitems; ++k) {
-      const int q = (int)(k % S);
-      if (k >= (size_t)S) {
-        // the consumers released this stage's previous item (use k / S - 1)
-        bool got = mbar_wait_bounded(&empty[q], (uint32_t)((k / S - 1) & 1), nullptr, 0.0);
-        got = __all_sync(0xffffffffu, got);
-        if (!got) {
-          ok = false;
-          break;
-        }
+  return st;
+}
+
+// the producer warp: items k .. k + nitems - 1 of the stream
+template <typename Issue>
+__device__ __forceinline__ bool stream_produce(const Stream& st, size_t& k, size_t nitems, Issue issue, double* err) {
+  const int lane = threadIdx.x & 31;
+  for (size_t m = 0; m < nitems; ++m, ++k) {
+    const int q = (int)(k % st.S);
+    if (k >= (size_t)st.S) {
+      // the consumers released this stage's previous item (use k / S - 1)
+      bool got = mbar_wait_bounded(&st.empty[q], (uint32_t)((k / st.S - 1) & 1), nullptr, 0.0);
+      got = __all_sync(0xffffffffu, got);
+      if (!got) {
+        if (lane == 0) *err = kErrWaitTimeout;
+        // items k - S .. k - 1 may still be in flight: wait for their copies
+        for (size_t f = k - st.S; f < k; ++f)
+          mbar_wait_bounded(&st.full[f % st.S], (uint32_t)((f / st.S) & 1), nullptr, 0.0);
+        return false;
       }
-      issue(k, buf + q * stage_stride, &full[q], lane);
     }
-    if (!ok) {
-      if (lane == 0) *err = kErrWaitTimeout;
-      // items k - S + 1 .. k - 1 may still be in flight: wait for their copies
-      const size_t lo = k >= (size_t)S ? k - S + 1 : 0;
-      for (size_t m = lo; m < k; ++m) mbar_wait_bounded(&full[m % S], (uint32_t)((m / S) & 1), nullptr, 0.0);
-    }
-  } else {  // consumers
-    for (size_t k = 0; k < nitems; ++k) {
-      const int q = (int)(k % S);
-      if (!mbar_wait_bounded(&full[q], (uint32_t)((k / S) & 1), err, kErrWaitTimeout)) break;
-      consume(k, buf + q * stage_stride);
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&empty[q]);
-    }
+    issue(m, st.buf + q * st.stride, &st.full[q], lane);
   }
-  __syncthreads();
+  return true;
+}
+
+// the consumer warps
+template <typename Consume>
+__device__ __forceinline__ bool stream_consume(const Stream& st, size_t& k, size_t nitems, Consume consume,
+                                               double* err) {
+  for (size_t m = 0; m < nitems; ++m, ++k) {
+    const int q = (int)(k % st.S);
+    bool got = mbar_wait_bounded(&st.full[q], (uint32_t)((k / st.S) & 1), err, kErrWaitTimeout);
+    got = __all_sync(0xffffffffu, got);
+    if (!got) return false;
+    consume(m, st.buf + q * st.stride);
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(&st.empty[q]);
+  }
+  return true;
+}
+
+// barrier of the consumer threads alone
+__device__ __forceinline__ void consumers_sync() {
+  asm volatile("bar.sync 1, %0;" ::"n"(kConsumerWarps * 32) : "memory");
 }
 
 // the producer lanes' share of an item: lane 0 announces the bytes, then copy c
@@ -696,42 +728,29 @@ __device__ __forceinline__ void issue_copies(uint64_t* bar, uint32_t bytes, int 
   for (int c = lane; c < ncopies; c += 32) copy_at(c);
 }
 
-// First pass, multi-dot: partial[b*ld + i0 + c] = sum over CTA b of V_{i0+c} . w
-// (w FP64, split on use) and, WITH_NORM, partial[b*ld + ncol_norm] = w . w.
-template <int CNT, bool WITH_NORM>
-__device__ __forceinline__ void multidot_df_stream(const float* __restrict__ Vf, int nvt, int i0,
-                                                   const double* __restrict__ w, size_t len,
-                                                   double* __restrict__ partial, int ncol_norm, int ld, int S,
-                                                   size_t stage_stride, double* err) {
+// First pass, multi-dot, of one chunk on the consumer threads: partial[b*ld + i0 + c] = sum over
+// CTA b of V_{i0+c} . w (w FP64, split on use) and, if `norm`, partial[b*ld + ld - 1] = w . w.
+// A stage holds the chunk's tiles and w's.  False when a wait ran out, now or before (!go: the
+// chunk is not read).
+template <int CNT>
+__device__ __forceinline__ bool multidot_df_chunk(const Stream& st, size_t& k, size_t mine, int i0, size_t len,
+                                                  double* __restrict__ partial, bool norm, int ld, bool go,
+                                                  double* err) {
   float s[CNT], er[CNT];
   double ww = 0.0;
 #pragma unroll
   for (int c = 0; c < CNT; ++c) s[c] = er[c] = 0.0f;
-  const size_t ntiles = (len + kTile - 1) / kTile;
-  const size_t mine = blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-  auto issue = [&](size_t k, unsigned char* st, uint64_t* bar, int lane) {
-    const size_t e0 = (blockIdx.x + k * gridDim.x) * (size_t)kTile;
-    const size_t n = len - e0 < (size_t)kTile ? len - e0 : (size_t)kTile;  // even: len is even
-    const uint32_t vb = (uint32_t)CNT * 2 * kTile * 4, db = (uint32_t)(n * 8);
-    // copy 0: the tile of vectors i0 .. i0 + CNT - 1 (contiguous); copy 1: w
-    issue_copies(bar, vb + db, 2, lane, [&](int c) {
-      if (c == 0)
-        bulk_copy_g2s(st, Vf + df_at(nvt, i0, e0, 0), vb, bar);
-      else
-        bulk_copy_g2s(st + vb, w + e0, db, bar);
-    });
-  };
   // thread t takes elements 2t and 2t + 1 of a tile (8-byte and 16-byte shared loads;
   // both lie inside or both beyond len, which is even)
-  auto consume = [&](size_t k, const unsigned char* st) {
-    const size_t e0 = (blockIdx.x + k * gridDim.x) * (size_t)kTile;
+  auto consume = [&](size_t m, const unsigned char* stage) {
+    const size_t e0 = (blockIdx.x + m * gridDim.x) * (size_t)kTile;
     if (e0 + 2 * threadIdx.x >= len) return;
-    const float2* sv = reinterpret_cast<const float2*>(st);
-    const double2 w2 = reinterpret_cast<const double2*>(st + (size_t)2 * CNT * kTile * 4)[threadIdx.x];
+    const float2* sv = reinterpret_cast<const float2*>(stage);
+    const double2 w2 = reinterpret_cast<const double2*>(stage + (size_t)2 * CNT * kTile * 4)[threadIdx.x];
     float wh0, wl0, wh1, wl1;
     split_f64(w2.x, wh0, wl0);
     split_f64(w2.y, wh1, wl1);
-    if (WITH_NORM) ww = fma(w2.y, w2.y, fma(w2.x, w2.x, ww));
+    if (norm) ww = fma(w2.y, w2.y, fma(w2.x, w2.x, ww));
 #pragma unroll
     for (int c = 0; c < CNT; ++c) {
       const float2 h = sv[(2 * c) * (kTile / 2) + threadIdx.x], l = sv[(2 * c + 1) * (kTile / 2) + threadIdx.x];
@@ -739,8 +758,9 @@ __device__ __forceinline__ void multidot_df_stream(const float* __restrict__ Vf,
       df_dot_acc(h.y, l.y, wh1, wl1, s[c], er[c]);
     }
   };
-  stream_items(mine, S, stage_stride, issue, consume, err);
-  __shared__ double red[kStreamThreads / 32][CNT + 1];
+  // a warp whose wait ran out goes on to the barriers, which the others reach as well
+  const bool ok = go && stream_consume(st, k, mine, consume, err);
+  __shared__ double red[kConsumerWarps][CNT + 1];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   {
     double t[CNT];
@@ -748,57 +768,87 @@ __device__ __forceinline__ void multidot_df_stream(const float* __restrict__ Vf,
     for (int c = 0; c < CNT; ++c) t[c] = f32_to_f64(s[c]) + f32_to_f64(er[c]);
     int c;
     const double v = warp_sums<CNT>(t, lane, c);
+    consumers_sync();  // the last chunk's sums have been read
     if (c < CNT) red[wid][c] = v;
   }
-  if (WITH_NORM) {
+  if (norm) {
     const double v = warp_sum(ww);
     if (lane == 0) red[wid][CNT] = v;
   }
-  __syncthreads();
-  if (threadIdx.x < CNT + (WITH_NORM ? 1 : 0)) {
+  consumers_sync();
+  if (threadIdx.x < CNT + (norm ? 1 : 0)) {
     double t = 0.0;
-    for (int q = 0; q < kStreamThreads / 32; ++q) t += red[q][threadIdx.x];
-    const int col = threadIdx.x < CNT ? i0 + threadIdx.x : ncol_norm;
+    for (int q = 0; q < kConsumerWarps; ++q) t += red[q][threadIdx.x];
+    const int col = threadIdx.x < CNT ? i0 + threadIdx.x : ld - 1;
     partial[(size_t)blockIdx.x * ld + col] = t;
   }
+  return ok;
 }
 
-template <int CNT, bool WITH_NORM>
-__global__ void __launch_bounds__(kStreamThreads, 1) multidot_df_kernel(const float* __restrict__ Vf, int nvt, int i0,
-                                                                        const double* __restrict__ w, size_t len,
-                                                                        double* __restrict__ partial, int nv, int ld,
-                                                                        int S, size_t stage_stride, double* err) {
-  multidot_df_stream<CNT, WITH_NORM>(Vf, nvt, i0, w, len, partial, nv, ld, S, stage_stride, err);
-}
-
-// device-resident index: nv = *jdev + 1 vectors; launch `chunk` of the balanced split
-// (exits when nv needs fewer chunks)
-template <bool WITH_NORM>
-__global__ void __launch_bounds__(kStreamThreads, 1) multidot_df_dyn_kernel(const float* __restrict__ Vf, int nvt,
-                                                                            int chunk, const double* __restrict__ w,
-                                                                            const int* __restrict__ jdev, size_t len,
-                                                                            double* __restrict__ partial, int ld,
-                                                                            int S, size_t stage_stride, double* err) {
-  const int nv = *jdev + 1;
-  if (chunk >= (nv + kChunk - 1) / kChunk) return;
-  if (!PC_DOK(nv < nvt && (len & 1) == 0, 201)) return;  // vector nv and the tiles exist
+// All nv vectors (jdev: nv = *jdev + 1) in one launch, chunk after chunk of the balanced split:
+// a launch a chunk cost a captured iteration the launches of chunks it has not reached, each
+// waiting for a whole SM's shared memory where several problems run, and every solve a
+// pipeline start.  The stages are sized for the largest chunk, the first.  Bound by HBM; two
+// CTAs an SM, so that two problems of a batch share it: eight problems of 31^2 x 16 to
+// 63^2 x 256 in one graph 21.1 -> 19.5 ms, 127^2 x 128 element solve 16.7 -> 16.5, 255^2 x 256
+// solve 0.5% faster, 63^3 x 128 0.8% slower than with one CTA, tiles of 512 and a launch a chunk.
+__global__ void __launch_bounds__(kStreamThreads, kStreamCtas)
+    multidot_df_kernel(const float* __restrict__ Vf, int nvt, int nv, const double* __restrict__ w,
+                       const int* __restrict__ jdev, size_t len, double* __restrict__ partial, bool norm, int ld,
+                       double* err) {
+  if (jdev) nv = *jdev + 1;
+  if (!PC_DOK(nv >= 1 && nv < nvt && (len & 1) == 0, 201)) return;  // vector nv and the tiles exist
+  const int nch = (nv + kChunk - 1) / kChunk;
+  const size_t ntiles = (len + kTile - 1) / kTile;
+  const size_t mine = blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
   int i0, cnt;
-  balanced_chunk(nv, chunk, &i0, &cnt);
-  switch (cnt) {
-#define PCOPT_DYN(k) \
-  case k: multidot_df_stream<k, WITH_NORM>(Vf, nvt, i0, w, len, partial, ld - 1, ld, S, stage_stride, err); break;
-    PCOPT_DYN(1) PCOPT_DYN(2) PCOPT_DYN(3) PCOPT_DYN(4) PCOPT_DYN(5) PCOPT_DYN(6) PCOPT_DYN(7) PCOPT_DYN(8)
-    PCOPT_DYN(9) PCOPT_DYN(10) PCOPT_DYN(11) PCOPT_DYN(12) PCOPT_DYN(13) PCOPT_DYN(14) PCOPT_DYN(15) PCOPT_DYN(16)
+  balanced_chunk(nv, 0, &i0, &cnt);
+  const size_t stride = stage_stride_of(cnt);
+  const Stream st = stream_begin(stream_stages_for(stride), stride);
+  size_t k = 0;
+  if (threadIdx.x >= kConsumerWarps * 32) {
+    for (int chunk = 0; chunk < nch; ++chunk) {
+      balanced_chunk(nv, chunk, &i0, &cnt);
+      auto issue = [&](size_t m, unsigned char* stage, uint64_t* bar, int lane) {
+        const size_t e0 = (blockIdx.x + m * gridDim.x) * (size_t)kTile;
+        const size_t n = len - e0 < (size_t)kTile ? len - e0 : (size_t)kTile;  // even: len is even
+        const uint32_t vb = (uint32_t)cnt * 2 * kTile * 4, db = (uint32_t)(n * 8);
+        // copy 0: the tile of vectors i0 .. i0 + cnt - 1 (contiguous); copy 1: w
+        issue_copies(bar, vb + db, 2, lane, [&](int c) {
+          if (c == 0)
+            bulk_copy_g2s(stage, Vf + df_at(nvt, i0, e0, 0), vb, bar);
+          else
+            bulk_copy_g2s(stage + vb, w + e0, db, bar);
+        });
+      };
+      if (!stream_produce(st, k, mine, issue, err)) break;
+    }
+  } else {
+    bool ok = true;
+    for (int chunk = 0; chunk < nch; ++chunk) {
+      balanced_chunk(nv, chunk, &i0, &cnt);
+      const bool nrm = norm && chunk == 0;
+      switch (cnt) {
+#define PCOPT_DYN(n) \
+  case n: \
+    ok = multidot_df_chunk<n>(st, k, mine, i0, len, partial, nrm, ld, ok, err); \
+    break;
+        PCOPT_DYN(1) PCOPT_DYN(2) PCOPT_DYN(3) PCOPT_DYN(4) PCOPT_DYN(5) PCOPT_DYN(6) PCOPT_DYN(7) PCOPT_DYN(8)
+        PCOPT_DYN(9) PCOPT_DYN(10) PCOPT_DYN(11) PCOPT_DYN(12) PCOPT_DYN(13) PCOPT_DYN(14) PCOPT_DYN(15)
+        PCOPT_DYN(16)
 #undef PCOPT_DYN
-    default: break;
+        default: break;
+      }
+    }
   }
+  __syncthreads();
 }
 
 // First pass, update: vector nv = (w - sum_{i < nv} coef_i V_i) * scale (double-float),
 // vf = its hi plane (contiguous), partial[b] = CTA sum of |w - sum|^2 (FP64, before
 // scaling).  The stream walks (tile, group of 16 vectors) items; w is copied with a
 // tile's first group.  With jdev: nv = *jdev + 1.
-__global__ void __launch_bounds__(kStreamThreads, 1) update_df_kernel(float* Vf, int nvt, int nv,
+__global__ void __launch_bounds__(kStreamThreads, kStreamCtas) update_df_kernel(float* Vf, int nvt, int nv,
                                                                       const double* __restrict__ coef,
                                                                       const double* __restrict__ w, float* vf,
                                                                       size_t len, const double* __restrict__ scale,
@@ -893,8 +943,13 @@ __global__ void __launch_bounds__(kStreamThreads, 1) update_df_kernel(float* Vf,
       reinterpret_cast<float2*>(vf + e0)[threadIdx.x] = make_float2(hv[0], hv[1]);
     }
   };
-  __syncthreads();  // coefficients staged
-  stream_items(mine * (size_t)G, S, stage_stride, issue, consume, err);
+  const Stream st = stream_begin(S, stage_stride);  // its barrier: the coefficients are staged
+  size_t item = 0;
+  if (threadIdx.x >= kConsumerWarps * 32)
+    stream_produce(st, item, mine * (size_t)G, issue, err);
+  else
+    stream_consume(st, item, mine * (size_t)G, consume, err);
+  __syncthreads();
   __shared__ double red[kStreamThreads / 32];
   acc = warp_sum(acc);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
@@ -907,9 +962,9 @@ __global__ void __launch_bounds__(kStreamThreads, 1) update_df_kernel(float* Vf,
 }
 
 // The second pass reads the hi planes directly, four consecutive elements of a vector a
-// thread (16-byte loads of 2 KB pieces, several vectors' in flight): 5.8 TB/s over the three
-// kernels at 255^2 x 256, 5.1 with one element a thread.  Bound by HBM.  `len` is even, so the last group may hold two elements: what lies beyond
-// len in the last tile is never used.
+// thread (16-byte loads of 1 KB pieces, several vectors' in flight): 5.8 TB/s over the three
+// kernels at 255^2 x 256, 5.1 with one element a thread.  Bound by HBM.  `len` is even, so the
+// last group may hold two elements: what lies beyond len in the last tile is never used.
 __device__ __forceinline__ float4 load_group(const float* p, bool whole) {
   float4 v = __ldg(reinterpret_cast<const float4*>(p));
   if (!whole) v.z = v.w = 0.0f;
@@ -964,12 +1019,13 @@ __global__ void __launch_bounds__(kThreads) multidot_lp_kernel(const float* __re
   multidot_lp_body<CNT>(Vf, nvt, i0, nv, len, partial, ld);
 }
 
-__global__ void __launch_bounds__(kThreads) multidot_lp_dyn_kernel(const float* __restrict__ Vf, int nvt, int i0,
+// captured iterations: blockIdx.y is the chunk of 16 vectors, those beyond nv = *jdev + 1 leave
+__global__ void __launch_bounds__(kThreads) multidot_lp_dyn_kernel(const float* __restrict__ Vf, int nvt,
                                                                    const int* __restrict__ jdev, size_t len,
                                                                    double* __restrict__ partial, int ld,
                                                                    const double* __restrict__ gate) {
   if (gated_off(gate)) return;
-  const int nv = *jdev + 1;
+  const int nv = *jdev + 1, i0 = (int)blockIdx.y * kChunk;
   if (i0 >= nv) return;
   if (!PC_DOK(nv < nvt, 205)) return;
   const int cnt = nv - i0 < kChunk ? nv - i0 : kChunk;
@@ -1149,18 +1205,10 @@ cudaError_t multidot_dispatch(int cnt, Launch& L, const double* V, size_t ldv, i
   }
 }
 
-size_t round128(size_t x) { return (x + 127) & ~(size_t)127; }
-
-// stages of `stride` bytes that fit the streaming CTA's shared-memory budget
-int stream_stages_for(size_t stride) {
-  const size_t s = (kStreamSmem - kBarBytes) / stride;
-  return (int)(s < 2 ? 2 : (s > 12 ? 12 : s));
-}
-
 // one streaming CTA per SM (the stages fill its shared memory), at most one per tile
 unsigned stream_grid(size_t len) {
   const size_t ntiles = (len + kTile - 1) / kTile;
-  const size_t sms = (size_t)num_sms();
+  const size_t sms = (size_t)num_sms() * kStreamCtas;
   return (unsigned)(ntiles < sms ? (ntiles ? ntiles : 1) : sms);
 }
 
@@ -1169,34 +1217,14 @@ cudaError_t allow_smem(K kern, size_t smem) {
   return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
-template <int CNT, bool N>
-cudaError_t multidot_df_chunk(Launch& L, const float* Vf, int nvt, int i0, const double* w, size_t len,
-                              double* partial, int nv, int ld, double* err, unsigned* blocks_out) {
-  const size_t stride = round128((size_t)2 * CNT * kTile * 4 + (size_t)kTile * 8);
-  const int S = stream_stages_for(stride);
-  const size_t smem = kBarBytes + S * stride;
-  auto kern = multidot_df_kernel<CNT, N>;
-  cudaError_t e = allow_smem(kern, smem);
+cudaError_t multidot_df_launch(Launch& L, const float* Vf, int nvt, int nv, const int* jdev, const double* w,
+                               size_t len, double* partial, bool norm, int ld, double* err, unsigned nb) {
+  cudaError_t e = allow_smem(multidot_df_kernel, kStreamSmem);
   if (e != cudaSuccess) return e;
-  const unsigned nb = stream_grid(len);
-  *blocks_out = nb;
+  const double nch = (nv + kChunk - 1) / kChunk;
   L.begin(KC_DOT);
-  kern<<<nb, kStreamThreads, smem, L.stream>>>(Vf, nvt, i0, w, len, partial, nv, ld, S, stride, err);
-  return L.end(KC_DOT, 8.0 * len * (CNT + 1), 2.0 * len * (CNT + (N ? 1 : 0)));
-}
-
-template <bool N>
-cudaError_t multidot_df_dispatch(int cnt, Launch& L, const float* Vf, int nvt, int i0, const double* w,
-                                 size_t len, double* partial, int nv, int ld, double* err, unsigned* nb) {
-  switch (cnt) {
-#define PCOPT_CASE(k) \
-  case k: return multidot_df_chunk<k, N>(L, Vf, nvt, i0, w, len, partial, nv, ld, err, nb);
-    PCOPT_CASE(1) PCOPT_CASE(2) PCOPT_CASE(3) PCOPT_CASE(4) PCOPT_CASE(5) PCOPT_CASE(6) PCOPT_CASE(7)
-    PCOPT_CASE(8) PCOPT_CASE(9) PCOPT_CASE(10) PCOPT_CASE(11) PCOPT_CASE(12) PCOPT_CASE(13) PCOPT_CASE(14)
-    PCOPT_CASE(15) PCOPT_CASE(16)
-#undef PCOPT_CASE
-    default: return cudaErrorInvalidValue;
-  }
+  multidot_df_kernel<<<nb, kStreamThreads, kStreamSmem, L.stream>>>(Vf, nvt, nv, w, jdev, len, partial, norm, ld, err);
+  return jdev ? L.end(KC_DOT, 0.0, 0.0) : L.end(KC_DOT, 8.0 * len * (nv + nch), 2.0 * len * (nv + (norm ? 1 : 0)));
 }
 
 template <int CNT>
@@ -1354,18 +1382,12 @@ cudaError_t launch_multidot_df(Launch& L, const float* Vf, int nvt, int nv, cons
       cg.nb[c] = nb;
       nb_sum += nb * (double)cnt;
     }
-  } else {  // balanced chunks, every one on the same streaming grid
-    const int nch = (nv + kChunk - 1) / kChunk;
-    unsigned nb = 0;
-    for (int c = 0; c < nch; ++c) {
-      int i0, cnt;
-      balanced_chunk(nv, c, &i0, &cnt);
-      cudaError_t e = (i0 == 0 && ww) ? multidot_df_dispatch<true>(cnt, L, Vf, nvt, i0, w, len, partial, nv, ld, err, &nb)
-                                      : multidot_df_dispatch<false>(cnt, L, Vf, nvt, i0, w, len, partial, nv, ld, err, &nb);
-      if (e != cudaSuccess) return e;
-      nb_sum += nb * (double)cnt;
-    }
+  } else {
+    const unsigned nb = stream_grid(len);
+    cudaError_t e = multidot_df_launch(L, Vf, nvt, nv, nullptr, w, len, partial, ww != nullptr, ld, err, nb);
+    if (e != cudaSuccess) return e;
     cg = one_grid(nb);
+    nb_sum = nb * (double)nv;
   }
   const int ncols = nv + (ww && !lp ? 1 : 0);
   const int kc = lp ? KC_REORTH : KC_REDUCE;
@@ -1390,7 +1412,7 @@ cudaError_t launch_update_df(Launch& L, float* Vf, int nvt, int nv, const double
     update_lp_kernel<<<nb, kThreads, 0, L.stream>>>(Vf, nvt, nv, coef, len, partial, gate, nullptr);
     e = L.end(KC_REORTH, 0.0, 0.0);
   } else {
-    const size_t stride = round128((size_t)2 * kGroup * kTile * 4 + (size_t)kTile * 8);
+    const size_t stride = stage_stride_of(kGroup);
     const int S = stream_stages_for(stride);
     const size_t smem = kBarBytes + S * stride;
     if ((e = allow_smem(update_df_kernel, smem)) != cudaSuccess) return e;
@@ -1436,32 +1458,16 @@ cudaError_t launch_multidot_df_dev(Launch& L, const float* Vf, int nvt, int nv_m
   if (lp) {
     const unsigned nb = wave_blocks(multidot_lp_dyn_kernel, 0, (len + 3) / 4);
     cg = one_grid(nb);
-    for (int i0 = 0; i0 < nv_max; i0 += kChunk) {
-      L.begin(kc);
-      multidot_lp_dyn_kernel<<<nb, kThreads, 0, L.stream>>>(Vf, nvt, i0, jdev, len, partial, ld, gate);
-      cudaError_t e = L.end(kc, 0.0, 0.0);
-      if (e != cudaSuccess) return e;
-    }
-  } else {
-    const size_t stride = round128((size_t)2 * kChunk * kTile * 4 + (size_t)kTile * 8);
-    const int S = stream_stages_for(stride);
-    const size_t smem = kBarBytes + S * stride;
-    cudaError_t e = allow_smem(multidot_df_dyn_kernel<true>, smem);
-    if (e == cudaSuccess) e = allow_smem(multidot_df_dyn_kernel<false>, smem);
+    L.begin(kc);
+    multidot_lp_dyn_kernel<<<dim3(nb, (unsigned)((nv_max + kChunk - 1) / kChunk)), kThreads, 0, L.stream>>>(
+        Vf, nvt, jdev, len, partial, ld, gate);
+    cudaError_t e = L.end(kc, 0.0, 0.0);
     if (e != cudaSuccess) return e;
+  } else {
     const unsigned nb = stream_grid(len);
     cg = one_grid(nb);
-    for (int c = 0; c < (nv_max + kChunk - 1) / kChunk; ++c) {
-      L.begin(kc);
-      if (c == 0 && ww)
-        multidot_df_dyn_kernel<true><<<nb, kStreamThreads, smem, L.stream>>>(Vf, nvt, c, w, jdev, len, partial, ld,
-                                                                            S, stride, err);
-      else
-        multidot_df_dyn_kernel<false><<<nb, kStreamThreads, smem, L.stream>>>(Vf, nvt, c, w, jdev, len, partial, ld,
-                                                                             S, stride, err);
-      e = L.end(kc, 0.0, 0.0);
-      if (e != cudaSuccess) return e;
-    }
+    cudaError_t e = multidot_df_launch(L, Vf, nvt, nv_max, jdev, w, len, partial, ww != nullptr, ld, err, nb);
+    if (e != cudaSuccess) return e;
   }
   L.begin(kc);
   reduce_partials_kernel<<<nv_max + (ww && !lp ? 1 : 0), kThreads, 0, L.stream>>>(partial, cg, ld, out,
@@ -1487,7 +1493,7 @@ cudaError_t launch_update_df_dev(Launch& L, float* Vf, int nvt, int nv_max, cons
     nb = wave_blocks(update_lp_kernel, 0, (len + 3) / 4);
     update_lp_kernel<<<nb, kThreads, 0, L.stream>>>(Vf, nvt, nv_max, coef, len, partial, gate, jdev);
   } else {
-    const size_t stride = round128((size_t)2 * kGroup * kTile * 4 + (size_t)kTile * 8);
+    const size_t stride = stage_stride_of(kGroup);
     const int S = stream_stages_for(stride);
     const size_t smem = kBarBytes + S * stride;
     if ((e = allow_smem(update_df_kernel, smem)) != cudaSuccess) return e;
@@ -1520,23 +1526,15 @@ cudaError_t launch_multidot_dev(Launch& L, const double* V, size_t ldv, int nv_m
   if (nv_max < 1 || nv_max > kChunk * kMaxChunks) return cudaErrorInvalidValue;
   const int ld = nv_max + 1;
   // gated launches are the re-orthogonalisation pass: FP32 products (see the file header)
-  auto plain = (gate && lp_reorth) ? multidot_dyn_kernel<false, true> : multidot_dyn_kernel<false, false>;
-  const unsigned nb_norm = wave_blocks(multidot_dyn_kernel<true>, 0, len);
-  const unsigned nb_plain = wave_blocks(plain, 0, len);
-  ChunkGrids cg = one_grid(nb_plain);
+  auto kern = (gate && lp_reorth) ? multidot_dyn_kernel<true> : multidot_dyn_kernel<false>;
+  const unsigned nb = wave_blocks(kern, 0, len);
+  const ChunkGrids cg = one_grid(nb);
   const int kc = gate ? KC_REORTH : KC_DOT;
-  for (int i0 = 0, c = 0; i0 < nv_max; i0 += kChunk, ++c) {
-    L.begin(kc);
-    if (i0 == 0 && ww) {
-      cg.nb[0] = nb_norm;
-      multidot_dyn_kernel<true><<<nb_norm, kThreads, 0, L.stream>>>(V, ldv, i0, wbase, wstride, jdev, len, partial,
-                                                                   ld, gate);
-    } else {
-      plain<<<nb_plain, kThreads, 0, L.stream>>>(V, ldv, i0, wbase, wstride, jdev, len, partial, ld, gate);
-    }
-    cudaError_t e = L.end(kc, 0.0, 0.0);
-    if (e != cudaSuccess) return e;
-  }
+  L.begin(kc);
+  kern<<<dim3(nb, (unsigned)((nv_max + kChunk - 1) / kChunk)), kThreads, 0, L.stream>>>(
+      V, ldv, wbase, wstride, jdev, len, partial, ld, ww != nullptr, gate);
+  cudaError_t e = L.end(kc, 0.0, 0.0);
+  if (e != cudaSuccess) return e;
   L.begin(kc);
   reduce_partials_kernel<<<nv_max + (ww ? 1 : 0), kThreads, 0, L.stream>>>(partial, cg, ld, out, ww, nv_max, gate,
                                                                           jdev, prep && ww ? kThenPrep : kThenNothing,
