@@ -100,6 +100,7 @@ __global__ void __launch_bounds__(256) tfft_forward_kernel(const Tin* __restrict
 
 template <typename Tc, typename TU, typename Tout>
 __global__ void __launch_bounds__(256) tfft_inverse_kernel(const TU* __restrict__ spec,
+                                                           const Tc* __restrict__ dpow,
                                                            const Tc* __restrict__ dinv,
                                                            const typename Cx<Tc>::t* __restrict__ tw,
                                                            Tout* __restrict__ w, int64_t ms, int n, int logn,
@@ -133,6 +134,10 @@ __global__ void __launch_bounds__(256) tfft_inverse_kernel(const TU* __restrict_
   }
   __syncthreads();
   fft_columns<Tc, true>(z, tw, n, TS);
+  // D^{-1} / (2n): a product with the table in FP64; in FP32 the exact 1 / (2n), then the division
+  // by D (see regfft.cuh on why FP32 keeps its operations)
+  const Tc inv_2n = Tc(0.5) / Tc(n);
+  auto unscale = [&](Tc y, int j) { return sizeof(Tc) == 4 ? (y * inv_2n) / dpow[j] : y * dinv[j]; };
   Tout* w1 = w;
   Tout* w2 = w + (int64_t)n * ms;
   for (int e = threadIdx.x; e < n * TS; e += blockDim.x) {
@@ -141,8 +146,8 @@ __global__ void __launch_bounds__(256) tfft_inverse_kernel(const TU* __restrict_
     const int64_t s = s0 + c;
     if (s >= ms) continue;
     const int jr = n - 1 - j;
-    const Tc wt1 = z[jr * TS + c].x * dinv[jr];  // J D^{-1} ifft(hat w1)
-    const Tc wt2 = z[j * TS + c].y * dinv[j];    // D^{-1} ifft(hat w2)
+    const Tc wt1 = unscale(z[jr * TS + c].x, jr);  // J D^{-1} ifft(hat w1)
+    const Tc wt2 = unscale(z[j * TS + c].y, j);    // D^{-1} ifft(hat w2)
     w1[(int64_t)j * ms + s] = cvt<Tout>(wt1 - wt2);   // step 4: [[I, -I], [I, I]]
     w2[(int64_t)j * ms + s] = cvt<Tout>(wt1 + wt2);
   }
@@ -884,7 +889,7 @@ cudaError_t launch_tfft_inverse(Launch& L, int64_t ms, int n, const TU* spec, co
   const double bytes = 2.0 * nf * ms * sizeof(TU) + 2.0 * n * ms * sizeof(Tout) + cbytes;
   const double flops = (double)ms * (5.0 * n * ilog2(n) + 4.0 * n);
   L.begin(KC_TFFT_INV);
-  tfft_inverse_kernel<Tc, TU, Tout><<<blocks, 256, smem, L.stream>>>(spec, dinv, tw, w, ms, n, ilog2(n), TS, fc);
+  tfft_inverse_kernel<Tc, TU, Tout><<<blocks, 256, smem, L.stream>>>(spec, dpow, dinv, tw, w, ms, n, ilog2(n), TS, fc);
   return L.end(KC_TFFT_INV, bytes, flops);
 }
 

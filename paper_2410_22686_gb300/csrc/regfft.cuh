@@ -15,7 +15,8 @@ __device__ __forceinline__ constexpr int brev_ct(int i) {
   return r;
 }
 
-// cos(2 pi q / 32) for q = 0..8
+// cos(2 pi q / 32) for q = 0..8; q = 8 as the FP64 cosine of the rounded pi / 2 (what the
+// host-made twiddle tables hold)
 template <typename T>
 __device__ __forceinline__ constexpr T cos32(int q) {
   switch (q) {
@@ -27,18 +28,20 @@ __device__ __forceinline__ constexpr T cos32(int q) {
     case 5: return T(0.55557023301960222474283081394853);
     case 6: return T(0.38268343236508977172845998403040);
     case 7: return T(0.19509032201612826784828486847702);
-    default: return T(0);
+    default: return T(6.123233995736766e-17);
   }
 }
 
-// In-place R-point DFT of registers (R <= 32), the twiddles compile-time constants, quarter
-// turns costing their two sums alone.  In FP64, whose unit bounds the transforms, a butterfly
+// In-place R-point DFT of registers (R <= 32), the twiddles compile-time constants.  In FP64,
+// whose unit bounds the transforms, quarter turns cost their two sums alone and a butterfly
 // with another twiddle takes six fused multiply-adds (a + w b in four, a - w b as
 // 2 a - (a + w b)) where a product and two sums take eight: 148 operations for 16 points
 // instead of 196 (preconditioner apply in FP64, 31^2: n = 256 2.24e-15 off against 2.26e-15
-// before).  In FP32, bound elsewhere, the sums follow the product: the fused form's error is
-// 1-2% larger there.  HALF_IN: inputs R/2.. are zero; HALF_OUT: only outputs 0..R/2-1 are
-// wanted.
+// before).  In FP32, bound elsewhere, every twiddle is a product followed by the sums, quarter
+// turns too (their cosine is 6e-17): the values of the twiddle tables, bit for bit.  A solve
+// preconditioned in FP32 stops where FP32 rounding, amplified by A, stands at rtol, so another
+// order of these operations moves its solution by up to rtol (at rtol = 1e-8, 63^2 x 64, by
+// 4e-9).  HALF_IN: inputs R/2.. are zero; HALF_OUT: only outputs 0..R/2-1 are wanted.
 template <int R, bool INV, bool HALF_IN = false, bool HALF_OUT = false, typename C>
 __device__ __forceinline__ void dft_regs(C (&x)[R]) {
   typedef decltype(C().x) T;
@@ -64,7 +67,7 @@ __device__ __forceinline__ void dft_regs(C (&x)[R]) {
         } else if (p == 0) {
           x[g + p] = a + b;
           if (!last) x[g + p + half] = a - b;
-        } else if (2 * p == half) {  // w = -i (forward), i (inverse)
+        } else if (sizeof(T) == 8 && 2 * p == half) {  // w = -i (forward), i (inverse)
           C t;
           t.x = INV ? -b.y : b.y;
           t.y = INV ? b.x : -b.x;
@@ -85,9 +88,9 @@ __device__ __forceinline__ void dft_regs(C (&x)[R]) {
               x[g + p + half].y = fma(T(2), a.y, -t.y);
             }
           } else {
-            t.x = wr;
-            t.y = wi;
-            t = cmul(t, b);
+            // rounded as the product with a twiddle from memory: constants may be contracted otherwise
+            t.x = fma(wr, b.x, -__fmul_rn(wi, b.y));
+            t.y = fma(wr, b.y, __fmul_rn(wi, b.x));
             x[g + p] = a + t;
             if (!last) x[g + p + half] = a - t;
           }
