@@ -6,13 +6,15 @@
 // x_j + x_{N-j} and the even ones only the differences: m^2 / 2 products a line instead of m^2.
 // The FP64 kernel is bound by them: 100^2 x 102 planes, an axis pass 344 us with all m^2
 // products and 216 with half of them (194 at the FP64 unit's rate), the fused last axis
-// 2 x 344 + 35 -> 452; FP32 102 -> 39 us.
+// 2 x 344 + 35 -> 452.  FP32, bound elsewhere, takes all m products of an output, j ascending:
+// a solve preconditioned in FP32 stops where FP32 rounding, amplified by A, stands at rtol, so
+// with sums and differences its solution moves by up to rtol (30^2 x 50 at rtol = 1e-8: 1e-8).
 //
 // A CTA of 256 threads holds a tile of lines in shared memory, the line index fastest; a
-// thread forms up to four outputs of one parity of its line at a time.  S is read through
-// L1 along its columns (S is symmetric), the lines of a tile sharing every value.  The last
-// axis of a solve runs fused: transform, division by sigma M + tau K on the sine modes,
-// transform.
+// thread forms up to four outputs (FP64: of one parity) of its line at a time.  S is read
+// through L1, the lines of a tile sharing every value: in FP64 along its columns (S is
+// symmetric), in FP32 along its rows.  The last axis of a solve runs fused: transform,
+// division by sigma M + tau K on the sine modes, transform.
 #include <algorithm>
 
 #include "common.cuh"
@@ -23,43 +25,60 @@ namespace {
 
 constexpr int kDstThreads = 256;
 
-// outputs i = par + 2 (t0 + q G), q < NQ, of line c from its sums or differences
+// FP64: sums and differences of a line's ends (see the file's head)
+template <typename Tc>
+constexpr bool dst_folds() {
+  return sizeof(Tc) == 8;
+}
+
+// Outputs of line c: folded, i = par + 2 (t0 + q G), q < NQ, from the line's sums or
+// differences; else i = t0 + q G (par = 0) from the line.
 template <typename Tc, int NQ>
 __device__ __forceinline__ void dst_outputs(const typename Cx<Tc>::t* src, typename Cx<Tc>::t* dst,
                                             const Tc* __restrict__ S, int m, int lc, int c, int par, int t0, int G) {
+  constexpr bool F = dst_folds<Tc>();
   Tc ar[NQ], ai[NQ];
 #pragma unroll
   for (int q = 0; q < NQ; ++q) ar[q] = ai[q] = Tc(0);
-  const int terms = par == 0 ? (m + 1) / 2 : m / 2;
-  const Tc* s = S + par + 2 * t0;
-  for (int j = 0; j < terms; ++j, s += m) {
+  const int terms = !F ? m : par == 0 ? (m + 1) / 2 : m / 2;
+  // S_ij of output q at s[q * apart]; the next j lies `step` on
+  const Tc* s = F ? S + par + 2 * t0 : S + (int64_t)t0 * m;
+  const int apart = F ? 2 * G : G * m, step = F ? m : 1;
+  for (int j = 0; j < terms; ++j, s += step) {
     const typename Cx<Tc>::t v = src[((par == 0 ? j : m - 1 - j) << lc) + c];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
-      const Tc w = __ldg(s + 2 * q * G);
+      const Tc w = __ldg(s + q * apart);
       ar[q] = fma(w, v.x, ar[q]);
       ai[q] = fma(w, v.y, ai[q]);
     }
   }
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) dst[((par + 2 * (t0 + q * G)) << lc) + c] = cmk<Tc>(ar[q], ai[q]);
+  for (int q = 0; q < NQ; ++q) {
+    const int i = F ? par + 2 * (t0 + q * G) : t0 + q * G;
+    dst[(i << lc) + c] = cmk<Tc>(ar[q], ai[q]);
+  }
 }
 
-// dst = DST-I of every line of src (which ends up as sums and differences).  Ends with a barrier.
+// dst = DST-I of every line of src (which ends up as sums and differences where the product
+// folds).  Ends with a barrier.
 template <typename Tc>
 __device__ __forceinline__ void dst_lines(typename Cx<Tc>::t* src, typename Cx<Tc>::t* dst, const Tc* __restrict__ S,
                                           int m, int lc) {
   typedef typename Cx<Tc>::t C;
+  constexpr bool F = dst_folds<Tc>();
   const int c = threadIdx.x & ((1 << lc) - 1), g = threadIdx.x >> lc, G = kDstThreads >> lc;
-  for (int j = g; j < m / 2; j += G) {
-    const C a = src[(j << lc) + c], b = src[((m - 1 - j) << lc) + c];
-    src[(j << lc) + c] = a + b;
-    src[((m - 1 - j) << lc) + c] = a - b;
+  if (F) {
+    for (int j = g; j < m / 2; j += G) {
+      const C a = src[(j << lc) + c], b = src[((m - 1 - j) << lc) + c];
+      src[(j << lc) + c] = a + b;
+      src[((m - 1 - j) << lc) + c] = a - b;
+    }
+    __syncthreads();
   }
-  __syncthreads();
 #pragma unroll
-  for (int par = 0; par < 2; ++par) {
-    const int cnt = (m - par + 1) / 2;  // outputs of this parity
+  for (int par = 0; par < (F ? 2 : 1); ++par) {
+    const int cnt = F ? (m - par + 1) / 2 : m;  // outputs (of this parity)
     for (int t0 = g; t0 < cnt; t0 += 4 * G) {
       switch (min(4, (cnt - t0 + G - 1) / G)) {
         case 4: dst_outputs<Tc, 4>(src, dst, S, m, lc, c, par, t0, G); break;
@@ -146,7 +165,7 @@ cudaError_t launch_dst_dense(Launch& L, const Grid& g, int planes, int axis, boo
   L.begin(kc);
   kern<<<(unsigned)((nlines + (1 << lc) - 1) >> lc), kDstThreads, smem, L.stream>>>(in, out, S, g.m, g.np, lstride,
                                                                                   nlines, lc, lamK, rmass, sigma);
-  return L.end(kc, 2.0 * tot * sizeof(C), (divide ? 2.0 : 1.0) * tot * 2.0 * g.m);
+  return L.end(kc, 2.0 * tot * sizeof(C), (divide ? 2.0 : 1.0) * tot * (dst_folds<Tc>() ? 2.0 : 4.0) * g.m);
 }
 
 template cudaError_t launch_dst_dense<float>(Launch&, const Grid&, int, int, bool, const float*, const float*,

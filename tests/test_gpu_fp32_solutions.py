@@ -13,8 +13,9 @@ from conftest import read_golden
 
 pytestmark = pytest.mark.gpu
 
-# register FFTs along time and space
-CASES = [(2, 31, 16, "fp32", 1e-8), (2, 31, 64, "fp32", 1e-8), (2, 31, 128, "fp32", 1e-8)]
+# register FFTs along time and space, dense sine products
+CASES = [(2, 31, 16, "fp32", 1e-8), (2, 31, 64, "fp32", 1e-8), (2, 31, 128, "fp32", 1e-8), (2, 45, 16, "fp32", 1e-8),
+         (2, 30, 8, "fp32", 1e-8)]
 
 
 def solution(d, m1, n, precision, gamma):
