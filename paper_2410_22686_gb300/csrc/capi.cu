@@ -186,7 +186,7 @@ struct pc_handle {
   // time FFT tables
   double* dpow64 = nullptr;  // eps^{j/n}
   float* dpow32 = nullptr;
-  double* dinv64 = nullptr;  // eps^{-j/n} / (2n)
+  double* dinv64 = nullptr;  // eps^{-j/n} / (2n); direct sums: / 2
   float* dinv32 = nullptr;
   double2* tw64 = nullptr;
   float2* tw32 = nullptr;
@@ -194,8 +194,8 @@ struct pc_handle {
   double2* sig1_64 = nullptr;  // the shift 1 (end-point solves)
   float2* sig1_32 = nullptr;
   float2* sig32 = nullptr;
-  void* cz_tab = nullptr;  // chirp-z table of the handle's precision (n not a power of two)
-  int cz_logM = 0;
+  void* cz_tab = nullptr;  // chirp-z table of the handle's precision
+  int cz_logM = 0;         // 0: n is a power of two or takes the direct sum
   // ideal RBD preconditioner (Eq. matrix_P): the real shift 1 + alpha of both planes
   int precond_kind = PC_PRECOND_EPS_CIRCULANT;
   int arnoldi = PC_ARNOLDI_AUTO;  // pc_arnoldi: basis storage and product precision of flexible GMRES
@@ -766,11 +766,15 @@ static int setup_impl(const pc_params* p, const double* a_nodes, void* krylov, s
   // ---- time FFT tables
   {
     const int n = h->n;
+    // lengths that are not powers of two: the chirp-z method, but for FP32 around exact spatial
+    // solves or BF16 storage (see k_tchirp.cu); the direct sums apply 1 / n themselves
+    h->cz_logM = h->fp32 && (spatial == PC_SPATIAL_FST || h->bf16s) ? 0 : chirp_log2(n);
+    const double ddiv = h->cz_logM || (n & (n - 1)) == 0 ? 2.0 * n : 2.0;
     // full circle of twiddles exp(-2 pi i k / n), k = 0..n-1
     std::vector<double> dp(n), di(n), twr(n), twi(n);
     for (int j = 0; j < n; ++j) {
       dp[j] = std::pow(p->eps, (double)j / n);
-      di[j] = std::pow(p->eps, -(double)j / n) / (2.0 * n);
+      di[j] = std::pow(p->eps, -(double)j / n) / ddiv;
     }
     for (int k = 0; k < n; ++k) {
       const double th = 2.0 * M_PI * (double)k / n;
@@ -801,8 +805,7 @@ static int setup_impl(const pc_params* p, const double* a_nodes, void* krylov, s
     if ((rc = upload_c(h, (void**)&h->sigP64, shiftP, zero2, false, st))) goto fail_out;
     if ((rc = upload_c(h, (void**)&h->sigP32, shiftP, zero2, true, st))) goto fail_out;
   }
-  if (chirp_log2(h->n)) {
-    h->cz_logM = chirp_log2(h->n);
+  if (h->cz_logM) {
     std::vector<double> re, im;
     chirp_table(h->n, h->cz_logM, re, im);
     if ((rc = upload_c(h, &h->cz_tab, re, im, h->fp32, st))) goto fail_out;
@@ -1306,7 +1309,7 @@ static cudaError_t precond_t(pc_handle* h, Launch& L, const Tin* v, Tout* w, siz
     if (stride != 0 || jdev != nullptr) return cudaErrorNotSupported;  // graph solves reject it first
     return precond_ideal_t<Tc, TU, Tout, Tin>(h, L, v, w);
   }
-  // n not a power of two: the chirp-z transforms (host-driven solves only, so no index)
+  // the chirp-z transforms: host-driven solves only, so no index
   const ChirpZ<Tc> cz{(const C*)h->cz_tab, h->cz_logM};
   if (cz.logM && jdev) return cudaErrorNotSupported;
   cudaError_t e = cz.logM ? launch_tchirp_forward<Tc, Tin>(L, h->ms, h->n, v, Tables<Tc>::dpow(h), cz, (C*)h->lv[0].r)

@@ -347,7 +347,7 @@ cudaError_t launch_fevar3_objective_grad(Launch& L, int m, int n, double h, doub
 
 // forward scaled time FFT: v (FP64 [2][n][ms]) -> spectral planes [2*nfreq][ms]
 // (twice the spectra: see k_tfft.cu)
-// dpow[j] = eps^{j/n}, dinv[j] = eps^{-j/n} / (2n), tw[k] = exp(-2 pi i k/n) for k = 0..n-1
+// dpow[j] = eps^{j/n}, dinv[j] = eps^{-j/n} / (2n) (direct sums: / 2), tw[k] = exp(-2 pi i k/n) for k = 0..n-1
 // With jdev != nullptr the input is v + (*jdev) * vstride (device-resident Arnoldi index).
 // input v: FP64 basis vectors, or (Tc = float) their FP32 rounding
 template <typename Tc, typename Tin = double>
@@ -373,7 +373,8 @@ cudaError_t launch_tfft_inverse(Launch& L, int64_t ms, int n, const TU* spec, co
                                 const int* jdev = nullptr, FineCorrection<TU> fc = FineCorrection<TU>());
 
 // Time transforms of lengths that are not powers of two by the chirp-z method
-// (k_tchirp.cu), n >= kChirpMinN (shorter ones take the direct sum of k_tfft.cu).  One
+// (k_tchirp.cu), n >= kChirpMinN (shorter ones, and FP32 ones around sine-transform solves,
+// take the direct sum of k_tfft.cu).  One
 // table: chirp c_j = exp(-pi i j^2 / n), j < n; filter = DFT_M(conj c) / M at
 // chirp_position; roots exp(-2 pi i q / M), q < M.  logM = 0: no table.
 constexpr int kChirpMinN = 24;

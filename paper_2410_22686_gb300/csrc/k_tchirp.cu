@@ -19,6 +19,11 @@
 // larger, n = 511 in FP32: 3.0e-6 against 1.4e-6).  31^2 columns, forward, FP64: n = 24
 // 53.5 -> 17.2 us, n = 31 71.9 -> 16.8, n = 100 343 -> 39, n = 511 2058 -> 162;
 // FP32: n = 24 12.6 -> 7.8, n = 100 77.9 -> 10.6, n = 511 391 -> 19.
+//
+// FP32 transforms around sine-transform solves keep the direct sum at every length: what such
+// a solve leaves at rtol is FP32 rounding amplified by A, and another order of the sums moves
+// its solution by up to rtol (31^2 x 63 at rtol = 1e-8: 9.5e-9).  Around multigrid the cycle's
+// own error is what is left there, and the solutions agree to 1e-12.
 #include <algorithm>
 
 #include "common.cuh"

@@ -13,7 +13,8 @@
 // hat v1[k], and both planes of a pair share sigma_k = lambda_k + alpha.  The two
 // parts of z carry the same scaling eps^{j/n} at every j, so the packing costs no
 // accuracy.  The planes hold twice these spectra: the 1/2 of the split and the 1/n of the
-// inverse transform (both exact for powers of two) are in the table dinv = eps^{-j/n} / (2n).
+// inverse transform (both exact for powers of two) are in the table dinv = eps^{-j/n} / (2n)
+// (direct sums: the 1/2 alone).
 // (Packing D^{-1} v1 with D v2 instead, the form C^T = D F conj(Lambda)
 // F^* D^{-1} suggests, mixes parts whose ratio reaches eps^{-2}: the smaller part then
 // keeps only about u / eps^2 of relative accuracy, which ruins an FP32 transform at
@@ -501,10 +502,10 @@ __global__ void __launch_bounds__(256) tfft4s_inverse_kernel(const TU* __restric
 }
 
 // ---------------------------------------------------------------------------
-// Direct DFT along time for short lengths that are not powers of two (n < kChirpMinN;
-// longer ones take the chirp-z method, k_tchirp.cu): a CTA holds TS columns of all n time samples in shared
-// memory and forms each needed frequency as a plain sum with the twiddle index
-// advanced incrementally modulo n.  n^2 work per column.
+// Direct DFT along time for lengths that are not powers of two and do not take the chirp-z
+// method of k_tchirp.cu: n < kChirpMinN, and FP32 around sine-transform solves.  A CTA holds
+// TS columns of all n time samples in shared memory and forms each needed frequency as a plain
+// sum with the twiddle index advanced incrementally modulo n.  n^2 work per column.
 template <typename Tc, typename Tin>
 __global__ void __launch_bounds__(256) tdft_forward_kernel(const Tin* __restrict__ v, const Tc* __restrict__ dpow,
                                                            const Tc* __restrict__ dinv,
@@ -583,6 +584,7 @@ __global__ void __launch_bounds__(256) tdft_inverse_kernel(const TU* __restrict_
     if (k > 0 && 2 * k < n) z[(n - k) * TS + c] = cmk<Tc>(sb.x + sa.y, sa.x - sb.y);
   }
   __syncthreads();
+  const Tc inv_n = Tc(1) / Tc(n);  // dinv carries the 1/2 of the split alone: its product with 1/n is not exact
   C* o = z + (size_t)n * TS;  // [n][TS]: half 1 in .x, half 2 in .y, both at their own time
   for (int e = threadIdx.x; e < n * TS; e += blockDim.x) {
     const int j = e / TS, c = e - (e / TS) * TS;
@@ -596,8 +598,8 @@ __global__ void __launch_bounds__(256) tdft_inverse_kernel(const TU* __restrict_
       ij += j;
       if (ij >= n) ij -= n;
     }
-    o[(n - 1 - j) * TS + c].x = dinv[j] * y.x;  // J D^{-1} ifft(hat w1)
-    o[j * TS + c].y = dinv[j] * y.y;            // D^{-1} ifft(hat w2)
+    o[(n - 1 - j) * TS + c].x = dinv[j] * (y.x * inv_n);  // J D^{-1} ifft(hat w1)
+    o[j * TS + c].y = dinv[j] * (y.y * inv_n);            // D^{-1} ifft(hat w2)
   }
   __syncthreads();
   Tout* w1 = w;

@@ -13,9 +13,10 @@ from conftest import read_golden
 
 pytestmark = pytest.mark.gpu
 
-# register FFTs along time and space, dense sine products
+# register FFTs along time and space, dense sine products,
+# direct sums along time, 3D
 CASES = [(2, 31, 16, "fp32", 1e-8), (2, 31, 64, "fp32", 1e-8), (2, 31, 128, "fp32", 1e-8), (2, 45, 16, "fp32", 1e-8),
-         (2, 30, 8, "fp32", 1e-8)]
+         (2, 30, 8, "fp32", 1e-8), (2, 31, 33, "fp32", 1e-8), (2, 30, 50, "fp32", 1e-8), (3, 15, 33, "fp32", 1e-8)]
 
 
 def solution(d, m1, n, precision, gamma):
