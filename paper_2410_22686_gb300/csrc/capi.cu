@@ -176,7 +176,7 @@ struct pc_handle {
 
   std::vector<LevelBuf> lv;
   int coarse_l0 = 0;                 // first level run by the fused coarse-cycle kernel
-  bool tail2 = false;                // 2D FP32 arithmetic: that kernel is mg_tail2 (from 63^2)
+  bool tail2 = false;                // 2D FP32 iterates: that kernel is mg_tail2 (from 63^2)
   Tiles tiles;                       // tile shapes of the tunable kernels (0 = default)
   float2* wdf = nullptr;             // level-0 face weights and diagonal as (hi, lo) float pairs
   float2* ddf = nullptr;
@@ -738,13 +738,11 @@ static int setup_impl(const pc_params* p, const double* a_nodes, void* krylov, s
       h->alpha_df = make_float2(ah, (float)(h->alpha - (double)ah));
     }
     // the fused lower cycle takes every level from the first with m <= 63 (2D, FP32
-    // arithmetic: one in-place array per level), 31 (2D, FP64 iterates) or 15 (3D).  With
-    // BF16 storage the levels from 63^2 down stay in FP32 there and are rounded once; they
-    // took a down leg, a coarse cycle from 31^2 and a prolongation before (127^2 x 64
-    // solve: 8.25 -> 7.60 ms).  (The in-place kernel also runs FP64 iterates, but one CTA of
-    // 133 KB per plane made the ideal preconditioner's two-plane steps slower: 29.6 -> 34.8
+    // iterates: one in-place array per level), 31 (2D, FP64 iterates or BF16 storage)
+    // or 15 (3D).  (The in-place kernel also runs FP64 iterates, but one CTA of 133 KB
+    // per plane made the ideal preconditioner's two-plane steps slower: 29.6 -> 34.8
     // ms per apply at 255^2 x 256.)
-    h->tail2 = dim == 2 && h->fp32 && !h->fevar;
+    h->tail2 = dim == 2 && h->fp32 && !h->bf16s && !h->fevar;
     // Element multigrid in 2D: from 63^2 in FP32 (74 KB of shared memory), 31^2 in FP64.
     const bool tail63 = h->tail2 || (h->fevar && dim == 2 && h->fp32);
     const int mthr = tail63 ? kMgTailMaxM : (dim == 2 ? 31 : 15);
@@ -1247,9 +1245,9 @@ static cudaError_t spatial_solve(pc_handle* h, Launch& L, int nplanes = 0,
   {
     const CoarseLevels<Tc>& cl = coarse_of<Tc>(h);
     bool done = false;
-    if constexpr (std::is_same<Tc, float>::value) {
+    if constexpr (std::is_same<Tc, float>::value && std::is_same<TU, float2>::value) {
       if (h->tail2) {
-        if ((e = launch_mg_tail2<TU>(L, P, cl, sig, (const C*)h->lv[l0].r, (TU*)h->lv[l0].u)) != cudaSuccess) return e;
+        if ((e = launch_mg_tail2(L, P, cl, sig, (const C*)h->lv[l0].r, (C*)h->lv[l0].u)) != cudaSuccess) return e;
         done = true;
       }
     }

@@ -481,9 +481,8 @@ cudaError_t launch_fe3_tail(Launch& L, int planes, const FeLevels<Tc>& lv, Tc ta
 // m <= kMgTailMaxM, one array per level updated in place (k_mgtail.cu)
 constexpr int kMgTailMaxM = 63;
 bool mg_tail2_supported(const CoarseLevels<float>& lv);
-template <typename TU>
 cudaError_t launch_mg_tail2(Launch& L, int planes, const CoarseLevels<float>& lv, const float2* sigma, const float2* r0,
-                            TU* u0);
+                            float2* u0);
 template <typename Tc, typename TU>
 size_t mg_coarse_cycle_smem(const CoarseLevels<Tc>& lv);
 template <typename Tc, typename TU>

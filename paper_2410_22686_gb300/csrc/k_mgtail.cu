@@ -1,7 +1,6 @@
 // Lower part of the 2D V(1,0) cycle (Section 2.1, step 2 of the apply of
 // P_eps^{-1}, variable a) in one launch: from the first level with at most 63^2
-// points down to the one-point level and back, for FP32 arithmetic (the iterate is rounded
-// to BF16 where it is stored so, once, at the end; FP64 handles keep
+// points down to the one-point level and back, for FP32 iterates (FP64 handles keep
 // the coarse-cycle kernel from 31^2: with FP64 values a plane needs one 133 KB CTA,
 // which made the two-plane steps of the ideal preconditioner slower).
 //
@@ -76,10 +75,10 @@ __device__ __forceinline__ typename Cx<Tc>::t red_residual(const typename Cx<Tc>
 // would otherwise keep the next point's loads behind it)
 constexpr int kTailBatch = 4;
 
-template <typename Tc, typename TU>
+template <typename Tc>
 __global__ void __launch_bounds__(tail_threads<Tc>(), sizeof(Tc) == 4 ? 2 : 1) mg_tail2_kernel(const CoarseLevels<Tc> lv,
                                                                       const typename Cx<Tc>::t* __restrict__ r0,
-                                                                      TU* __restrict__ u0,
+                                                                      typename Cx<Tc>::t* __restrict__ u0,
                                                                       const typename Cx<Tc>::t* __restrict__ sigma,
                                                                       int stage0) {
   typedef typename Cx<Tc>::t C;
@@ -272,9 +271,9 @@ __global__ void __launch_bounds__(tail_threads<Tc>(), sizeof(Tc) == 4 ? 2 : 1) m
     }
     __syncthreads();
   }
-  TU* dst = u0 + (int64_t)p * np0;
+  C* dst = u0 + (int64_t)p * np0;
 #pragma unroll 4
-  for (int s = tid; s < np0; s += NT) stc(dst, s, A[0][s]);
+  for (int s = tid; s < np0; s += NT) dst[s] = A[0][s];
 }
 
 template <typename Tc>
@@ -303,9 +302,8 @@ bool mg_tail2_supported(const CoarseLevels<float>& lv) {
   return lv.m[lv.count - 1] == 1;
 }
 
-template <typename TU>
 cudaError_t launch_mg_tail2(Launch& L, int planes, const CoarseLevels<float>& lv, const float2* sigma, const float2* r0,
-                            TU* u0) {
+                            float2* u0) {
   typedef float Tc;
   if (!mg_tail2_supported(lv) || planes < 1) return cudaErrorInvalidValue;
   // stage the first level's coefficients too when two CTAs still fit on an SM
@@ -313,18 +311,14 @@ cudaError_t launch_mg_tail2(Launch& L, int planes, const CoarseLevels<float>& lv
   const size_t all = base + tail_coef_smem<Tc>(lv, 0) - tail_coef_smem<Tc>(lv, 1);
   const int stage0 = all <= 100 * 1024 ? 1 : 0;
   const size_t smem = stage0 ? all : base;
-  cudaError_t e = cudaFuncSetAttribute(mg_tail2_kernel<Tc, TU>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(mg_tail2_kernel<Tc>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   double pts = 0;
   for (int l = 0; l < lv.count; ++l) pts += (double)lv.np[l];
   const double cs = sizeof(float2);
   L.begin(KC_MG_COARSE);
-  mg_tail2_kernel<Tc, TU><<<planes, tail_threads<Tc>(), smem, L.stream>>>(lv, r0, u0, sigma, stage0);
-  return L.end(KC_MG_COARSE, (double)planes * lv.np[0] * (cs + sizeof(TU)), (double)planes * pts * 60.0);
+  mg_tail2_kernel<Tc><<<planes, tail_threads<Tc>(), smem, L.stream>>>(lv, r0, u0, sigma, stage0);
+  return L.end(KC_MG_COARSE, (double)planes * lv.np[0] * 2.0 * cs, (double)planes * pts * 60.0);
 }
-template cudaError_t launch_mg_tail2<float2>(Launch&, int, const CoarseLevels<float>&, const float2*, const float2*,
-                                             float2*);
-template cudaError_t launch_mg_tail2<__nv_bfloat162>(Launch&, int, const CoarseLevels<float>&, const float2*,
-                                                     const float2*, __nv_bfloat162*);
 
 }  // namespace pcopt

@@ -1,9 +1,10 @@
-"""Solutions of solves preconditioned in FP32, against stored ones (GB300).  Where the spatial
-solve is exact, FP32 rounding amplified by A is all that is left of the residual at rtol; so the
-solution below rtol is what the order of the preconditioner's FP32 operations makes it.  Any
-other order is as accurate, but moves solutions by up to rtol (1e-8) from one version to the
-next; with these operations kept they agree to 1e-10 (the FP64 sums of an iteration may round
-otherwise).  1e-9 is between the two."""
+"""Solutions of solves preconditioned in FP32 or with BF16 storage, against stored ones (GB300).
+Where the spatial solve is exact, FP32 rounding amplified by A is all that is left of the
+residual at rtol, and BF16 storage rounds at 2^-9; so the solution below rtol is what the order
+of the preconditioner's FP32 operations makes it.  Any other order is as accurate, but moves
+solutions by up to rtol (1e-8) from one version to the next; with these operations kept they
+agree to 1e-10 (BF16: 3e-10; the FP64 sums of an iteration may round otherwise).  1e-9 is
+between the two."""
 import numpy as np
 import pytest
 import torch
@@ -14,9 +15,11 @@ from conftest import read_golden
 pytestmark = pytest.mark.gpu
 
 # register FFTs along time and space, dense sine products,
-# direct sums along time, 3D
+# direct sums along time, 3D;
+# levels stored in BF16
 CASES = [(2, 31, 16, "fp32", 1e-8), (2, 31, 64, "fp32", 1e-8), (2, 31, 128, "fp32", 1e-8), (2, 45, 16, "fp32", 1e-8),
-         (2, 30, 8, "fp32", 1e-8), (2, 31, 33, "fp32", 1e-8), (2, 30, 50, "fp32", 1e-8), (3, 15, 33, "fp32", 1e-8)]
+         (2, 30, 8, "fp32", 1e-8), (2, 31, 33, "fp32", 1e-8), (2, 30, 50, "fp32", 1e-8), (3, 15, 33, "fp32", 1e-8),
+         (2, 31, 64, "bf16s", 1e-8), (2, 31, 33, "bf16s", 1e-8)]
 
 
 def solution(d, m1, n, precision, gamma):
