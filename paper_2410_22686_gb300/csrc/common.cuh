@@ -622,6 +622,15 @@ cudaError_t launch_grad_chunked(Launch& L, const Grid& g, int n, double scale, c
                                 const double* lam, double* partial, int tj, double* grad);
 
 int num_sms();
+// Before a launch with `smem` bytes of dynamic shared memory.  The limit a kernel carries belongs
+// to the process, and handles are used from several threads: it is raised once, to all the
+// device gives, and never lowered (a limit set to each call's own size let another thread's
+// smaller one refuse the launch in between).  Sizes beyond it are refused.
+cudaError_t raise_dynamic_smem(const void* kern, size_t smem);
+template <typename K>
+cudaError_t allow_dynamic_smem(K kern, size_t smem) {
+  return raise_dynamic_smem(reinterpret_cast<const void*>(kern), smem);
+}
 // time blocks per thread of a double-float product launched with `blocks` CTAs per chunk of
 // time, for at least per_sm CTAs an SM (k_matvec.cu); tuned > 0 overrides
 int time_chunk_filling(int64_t blocks, int n, int per_sm, int tuned);

@@ -158,7 +158,7 @@ cudaError_t launch_dst_dense(Launch& L, const Grid& g, int planes, int axis, boo
   while (lc > 0 && (smem_of(lc) > 56 * 1024 || (lc > 1 && (nlines >> lc) < 2 * num_sms()))) --lc;
   const size_t smem = smem_of(lc);
   auto kern = divide ? dst_dense_kernel<Tc, true> : dst_dense_kernel<Tc, false>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
   const double tot = (double)planes * (double)g.np;
   const int kc = divide ? KC_FST_DIVIDE : KC_FST_AXIS;

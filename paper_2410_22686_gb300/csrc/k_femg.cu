@@ -349,7 +349,7 @@ cudaError_t launch_fe_down(Launch& L, int m, int planes, Tc h2, Tc tau, const Tc
   const int cy = fe_down_rows<Tc>(m, planes), mc = (m - 1) / 2;
   if (cy < 1) return cudaErrorInvalidValue;
   const size_t smem = fe_down_smem<Tc>(m, cy);
-  cudaError_t e = cudaFuncSetAttribute(fe_down_kernel<Tc>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(fe_down_kernel<Tc>, smem);
   if (e != cudaSuccess) return e;
   const double cs = sizeof(typename Cx<Tc>::t), np = (double)m * m * planes;
   L.begin(KC_MG_DOWN);
@@ -369,7 +369,7 @@ template <typename Tc>
 cudaError_t launch_fe_tail(Launch& L, int planes, const FeLevels<Tc>& lv, Tc tau, const typename Cx<Tc>::t* sigma,
                            const typename Cx<Tc>::t* r, typename Cx<Tc>::t* u) {
   const size_t smem = fe_tail_smem(lv);
-  cudaError_t e = cudaFuncSetAttribute(fe_tail_kernel<Tc>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(fe_tail_kernel<Tc>, smem);
   if (e != cudaSuccess) return e;
   const double cs = sizeof(typename Cx<Tc>::t), np = (double)lv.m[0] * lv.m[0] * planes;
   L.begin(KC_MG_COARSE);

@@ -423,10 +423,8 @@ cudaError_t launch_fe3_down(Launch& L, int m, int planes, Tc h, Tc tau, const Tc
   {
     const int cy = fe3_longest(m, 16, fe3_odd_smem<Tc>);
     const size_t odd = fe3_odd_smem<Tc>(m, cy), even = odd / 3;
-    if ((e = cudaFuncSetAttribute(fe3_layer_kernel<Tc, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)even)) !=
-            cudaSuccess ||
-        (e = cudaFuncSetAttribute(fe3_layer_kernel<Tc, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)odd)) !=
-            cudaSuccess)
+    if ((e = allow_dynamic_smem(fe3_layer_kernel<Tc, 0>, even)) != cudaSuccess ||
+        (e = allow_dynamic_smem(fe3_layer_kernel<Tc, 1>, odd)) != cudaSuccess)
       return e;
     // even rows 0, 2, .., m - 1 in strips of 2 cy rows (the last even row needs no strip of its own)
     const unsigned ns = (unsigned)std::max(1, (mc + cy - 1) / cy);
@@ -439,9 +437,7 @@ cudaError_t launch_fe3_down(Launch& L, int m, int planes, Tc h, Tc tau, const Tc
   }
   const int cy = fe3_longest(m, 8, fe3_restrict_smem<Tc>);
   const size_t smem = fe3_restrict_smem<Tc>(m, cy);
-  if ((e = cudaFuncSetAttribute(fe3_restrict_kernel<Tc>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-      cudaSuccess)
-    return e;
+  if ((e = allow_dynamic_smem(fe3_restrict_kernel<Tc>, smem)) != cudaSuccess) return e;
   L.begin(KC_MG_RESID_RESTRICT);
   fe3_restrict_kernel<Tc><<<dim3((unsigned)((mc + cy - 1) / cy), (unsigned)mc, (unsigned)planes), kFe3Threads, smem,
                             L.stream>>>(u, rc, E, sigma, m, h, tau, cy);
@@ -455,7 +451,7 @@ cudaError_t launch_fe3_tail(Launch& L, int planes, const FeLevels<Tc>& lv, Tc ta
   size_t n = (size_t)lv.m[0] * lv.m[0] * lv.m[0];
   for (int l = 0; l < lv.count; ++l) n += (size_t)lv.m[l] * lv.m[l] * lv.m[l];
   const size_t smem = n * sizeof(C);
-  cudaError_t e = cudaFuncSetAttribute(fe3_tail_kernel<Tc>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(fe3_tail_kernel<Tc>, smem);
   if (e != cudaSuccess) return e;
   const double np = (double)lv.m[0] * lv.m[0] * lv.m[0] * planes;
   L.begin(KC_MG_COARSE);

@@ -373,7 +373,7 @@ cudaError_t fst4s(Launch& L, const Grid& g, int64_t lstride, int64_t nlines, Tc 
   constexpr int COLS = 256 / N1;
   const size_t smem = ((size_t)(N1 + 1) * N2 * COLS + (size_t)g.m * COLS) * sizeof(typename Cx<Tc>::t);
   auto kern = fst4s_kernel<Tc, N1, N2, DIVIDE, HALF>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem)) != cudaSuccess) return e;
@@ -392,7 +392,7 @@ cudaError_t fst4_nt(Launch& L, const Grid& g, bool divide, int64_t lstride, int6
   const size_t smem = (size_t)(N1 + 1) * N2 * COLS * sizeof(typename Cx<Tc>::t);
   const unsigned blocks = (unsigned)((nlines + COLS - 1) / COLS);
   auto kern = divide ? fst4_kernel<Tc, N1, N2, true, HALF, NT> : fst4_kernel<Tc, N1, N2, false, HALF, NT>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
   kern<<<blocks, NT, smem, L.stream>>>(in, out, tw, g.m, g.np, lstride, nlines, hs, lamK, rmass, sigma);
   return cudaGetLastError();

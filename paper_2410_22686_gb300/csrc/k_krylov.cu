@@ -26,7 +26,10 @@
 // sums (warp shuffles, then shared memory) and a second kernel adds them in a
 // fixed order.  The multi-dot is instantiated per vector count (1..16) so that
 // every FMA it issues is useful; more vectors take several chunked launches.
+#include <map>
+#include <mutex>
 #include <type_traits>
+#include <utility>
 
 #include "common.cuh"
 #include "tma.cuh"
@@ -1212,14 +1215,9 @@ unsigned stream_grid(size_t len) {
   return (unsigned)(ntiles < sms ? (ntiles ? ntiles : 1) : sms);
 }
 
-template <typename K>
-cudaError_t allow_smem(K kern, size_t smem) {
-  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-
 cudaError_t multidot_df_launch(Launch& L, const float* Vf, int nvt, int nv, const int* jdev, const double* w,
                                size_t len, double* partial, bool norm, int ld, double* err, unsigned nb) {
-  cudaError_t e = allow_smem(multidot_df_kernel, kStreamSmem);
+  cudaError_t e = allow_dynamic_smem(multidot_df_kernel, kStreamSmem);
   if (e != cudaSuccess) return e;
   const double nch = (nv + kChunk - 1) / kChunk;
   L.begin(KC_DOT);
@@ -1415,7 +1413,7 @@ cudaError_t launch_update_df(Launch& L, float* Vf, int nvt, int nv, const double
     const size_t stride = stage_stride_of(kGroup);
     const int S = stream_stages_for(stride);
     const size_t smem = kBarBytes + S * stride;
-    if ((e = allow_smem(update_df_kernel, smem)) != cudaSuccess) return e;
+    if ((e = allow_dynamic_smem(update_df_kernel, smem)) != cudaSuccess) return e;
     nb = stream_grid(len);
     L.begin(KC_UPDATE);
     update_df_kernel<<<nb, kStreamThreads, smem, L.stream>>>(Vf, nvt, nv, coef, w, vf, len, scale, partial, nullptr, S,
@@ -1496,7 +1494,7 @@ cudaError_t launch_update_df_dev(Launch& L, float* Vf, int nvt, int nv_max, cons
     const size_t stride = stage_stride_of(kGroup);
     const int S = stream_stages_for(stride);
     const size_t smem = kBarBytes + S * stride;
-    if ((e = allow_smem(update_df_kernel, smem)) != cudaSuccess) return e;
+    if ((e = allow_dynamic_smem(update_df_kernel, smem)) != cudaSuccess) return e;
     nb = stream_grid(len);
     update_df_kernel<<<nb, kStreamThreads, smem, L.stream>>>(Vf, nvt, nv_max, coef, w, vf, len, scale, partial, jdev,
                                                             S, stride, err);
@@ -1604,6 +1602,26 @@ template cudaError_t launch_xupdate_dev<double>(Launch&, const double*, size_t, 
                                                 double*, size_t);
 template cudaError_t launch_xupdate_dev<float>(Launch&, const float*, size_t, int, const int*, const double*, double*,
                                                size_t);
+
+cudaError_t raise_dynamic_smem(const void* kern, size_t smem) {
+  static std::mutex mu;
+  static std::map<std::pair<int, const void*>, size_t> limits;  // one entry a kernel and device
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mu);
+  auto at = limits.find({dev, kern});
+  if (at == limits.end()) {
+    cudaFuncAttributes fa{};
+    int most = 0;
+    if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+    const int room = most - (int)fa.sharedSizeBytes;
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, room)) != cudaSuccess) return e;
+    at = limits.emplace(std::make_pair(dev, kern), (size_t)room).first;
+  }
+  return smem <= at->second ? cudaSuccess : cudaErrorInvalidValue;
+}
 
 int num_sms() {
   static int cached = 0;

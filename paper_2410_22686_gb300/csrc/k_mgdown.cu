@@ -461,8 +461,7 @@ cudaError_t down2(Launch& L, int m, int planes, int pch, const Tc* w, const Tc* 
   constexpr int WR = 2 * CX + 5;
   constexpr int NH = WR * ((WR + 1) / 2);  // slots per colour
   const size_t smem = (size_t)NH * (2 * sizeof(typename W4<Tc>::t) + 4 * sizeof(C) + 2 * sizeof(Tc));
-  cudaError_t e = cudaFuncSetAttribute(mg_down2_kernel<Tc, TU, CX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = allow_dynamic_smem(mg_down2_kernel<Tc, TU, CX>, smem);
   if (e != cudaSuccess) return e;
   // prefer shared memory in the unified L1 (the window is 50 KB per CTA in FP32)
   e = cudaFuncSetAttribute(mg_down2_kernel<Tc, TU, CX>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);

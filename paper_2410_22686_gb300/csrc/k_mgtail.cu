@@ -311,7 +311,7 @@ cudaError_t launch_mg_tail2(Launch& L, int planes, const CoarseLevels<float>& lv
   const size_t all = base + tail_coef_smem<Tc>(lv, 0) - tail_coef_smem<Tc>(lv, 1);
   const int stage0 = all <= 100 * 1024 ? 1 : 0;
   const size_t smem = stage0 ? all : base;
-  cudaError_t e = cudaFuncSetAttribute(mg_tail2_kernel<Tc>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(mg_tail2_kernel<Tc>, smem);
   if (e != cudaSuccess) return e;
   double pts = 0;
   for (int l = 0; l < lv.count; ++l) pts += (double)lv.np[l];

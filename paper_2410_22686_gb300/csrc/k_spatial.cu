@@ -888,9 +888,9 @@ cudaError_t launch_mg_coarse_cycle(Launch& L, int dim, int planes, const CoarseL
   const size_t smem = base + (stage ? coef : 0);
   cudaError_t e;
   if (dim == 2)
-    e = cudaFuncSetAttribute(mg_coarse_cycle_kernel<Tc, TU, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_dynamic_smem(mg_coarse_cycle_kernel<Tc, TU, 2>, smem);
   else
-    e = cudaFuncSetAttribute(mg_coarse_cycle_kernel<Tc, TU, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_dynamic_smem(mg_coarse_cycle_kernel<Tc, TU, 3>, smem);
   if (e != cudaSuccess) return e;
   double pts = 0;
   for (int l = 0; l < lv.count; ++l) pts += (double)lv.np[l];

@@ -294,7 +294,7 @@ cudaError_t launch_tchirp_forward(Launch& L, int64_t ms, int n, const Tin* v, co
   const int lc = cz_lc<Tc>(cz.logM, ms);
   const size_t smem = sizeof(C) << (cz.logM + lc);
   auto kern = tchirp_forward_kernel<Tc, Tin>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
   L.begin(KC_TFFT_FWD);
   kern<<<(unsigned)((ms + (1 << lc) - 1) >> lc), kCzThreads, smem, L.stream>>>(v, dpow, cz, spec, ms, n, lc);
@@ -309,7 +309,7 @@ cudaError_t launch_tchirp_inverse(Launch& L, int64_t ms, int n, const TU* spec, 
   const int lc = cz_lc<Tc>(cz.logM, ms);
   const size_t smem = sizeof(C) << (cz.logM + lc);
   auto kern = tchirp_inverse_kernel<Tc, TU, Tout>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
   const double cbytes = fc.ec ? (double)(n / 2 + 1) * 2.0 * fc.npc * sizeof(TU) : 0.0;
   L.begin(KC_TFFT_INV);

@@ -653,12 +653,12 @@ cudaError_t fwd4_nt(Launch& L, int64_t ms, const Tin* v, const Tc* dpow, const T
   const unsigned blocks = (unsigned)((ms + COLS - 1) / COLS);
   if constexpr (tfft_fp64_blocks<Tc, N1 * N2>() == 2) {
     auto kern = tfft4_forward_f64_kernel<Tin, N1, N2, NT>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<blocks, NT, smem, L.stream>>>(v, dpow, dinv, tw, spec, ms, vstride, jdev);
   } else {
     auto kern = tfft4_forward_kernel<Tin, Tc, N1, N2, NT>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<blocks, NT, smem, L.stream>>>(v, dpow, dinv, tw, spec, ms, vstride, jdev);
   }
@@ -680,7 +680,7 @@ cudaError_t inv4_nt(Launch& L, int64_t ms, const TU* spec, const Tc* dpow, const
   constexpr int COLS = NT / N1;
   const size_t smem = (size_t)N1 * N2 * COLS * sizeof(typename Cx<Tc>::t);
   auto kern = tfft4_inverse_kernel<Tc, TU, Tout, N1, N2, NT>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
   kern<<<(unsigned)((ms + COLS - 1) / COLS), NT, smem, L.stream>>>(spec, dpow, dinv, tw, w, ms, wstride, jdev, fc);
   return cudaGetLastError();
@@ -705,7 +705,7 @@ cudaError_t fwd4s(Launch& L, int64_t ms, const Tin* v, const Tc* dpow, const Tc*
   const size_t smem = (size_t)2 * 2 * n * COLS * sizeof(Tin) + (size_t)n * COLS * sizeof(typename Cx<Tc>::t);
   if (smem > 227 * 1024) return fwd4<Tin, Tc, N1, N2>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev);
   auto kern = tfft4s_forward_kernel<Tin, Tc, N1, N2>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem)) != cudaSuccess) return e;
@@ -726,7 +726,7 @@ cudaError_t inv4s(Launch& L, int64_t ms, const TU* spec, const Tc* dpow, const T
                       (size_t)n * COLS * sizeof(typename Cx<Tc>::t);
   if (smem > 227 * 1024) return inv4<Tc, TU, Tout, N1, N2>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc);
   auto kern = tfft4s_inverse_kernel<Tc, TU, Tout, N1, N2>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem)) != cudaSuccess) return e;
@@ -822,7 +822,7 @@ cudaError_t launch_tfft_forward(Launch& L, int64_t ms, int n, const Tin* v, cons
   if (!pow2) {
     const int TS = pick_ts_dft<Tc>(n);
     const size_t smem = (size_t)n * TS * sizeof(typename Cx<Tc>::t);
-    cudaError_t e = cudaFuncSetAttribute(tdft_forward_kernel<Tc, Tin>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(tdft_forward_kernel<Tc, Tin>, smem);
     if (e != cudaSuccess) return e;
     const int nf = n / 2 + 1;
     L.begin(KC_TFFT_FWD);
@@ -840,7 +840,7 @@ cudaError_t launch_tfft_forward(Launch& L, int64_t ms, int n, const Tin* v, cons
   }
   const int TS = pick_ts<Tc>(n);
   const size_t smem = (size_t)n * TS * sizeof(typename Cx<Tc>::t);
-  cudaError_t e = cudaFuncSetAttribute(tfft_forward_kernel<Tc, Tin>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(tfft_forward_kernel<Tc, Tin>, smem);
   if (e != cudaSuccess) return e;
   const unsigned blocks = (unsigned)((ms + TS - 1) / TS);
   const int nf = n / 2 + 1;
@@ -863,8 +863,7 @@ cudaError_t launch_tfft_inverse(Launch& L, int64_t ms, int n, const TU* spec, co
     const int TS = pick_ts_dft<Tc>(n);
     // the spectrum and, after the sums, both halves at their own times: two [n][TS] arrays
     const size_t smem = 2 * (size_t)n * TS * sizeof(typename Cx<Tc>::t);
-    cudaError_t e =
-        cudaFuncSetAttribute(tdft_inverse_kernel<Tc, TU, Tout>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(tdft_inverse_kernel<Tc, TU, Tout>, smem);
     if (e != cudaSuccess) return e;
     const int nf = n / 2 + 1;
     L.begin(KC_TFFT_INV);
@@ -883,8 +882,7 @@ cudaError_t launch_tfft_inverse(Launch& L, int64_t ms, int n, const TU* spec, co
   }
   const int TS = pick_ts<Tc>(n);
   const size_t smem = (size_t)n * TS * sizeof(typename Cx<Tc>::t);
-  cudaError_t e =
-      cudaFuncSetAttribute(tfft_inverse_kernel<Tc, TU, Tout>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(tfft_inverse_kernel<Tc, TU, Tout>, smem);
   if (e != cudaSuccess) return e;
   const unsigned blocks = (unsigned)((ms + TS - 1) / TS);
   const int nf = n / 2 + 1;
