@@ -552,7 +552,9 @@ static void chirp_table(int n, int b, std::vector<double>& re, std::vector<doubl
 // unknown) and of the preconditioned vectors Z (cap vectors, FP32 or FP64), each
 // part rounded up to 256 bytes; Z follows V
 static size_t round256(size_t b) { return (b + 255) / 256 * 256; }
-static size_t krylov_v_bytes(size_t U, int cap) { return round256((size_t)(cap + 1) * ((U + 511) / 512 * 512) * 8); }
+// doubles of one basis vector: U, or its two FP32 planes, in whole tiles
+static size_t basis_stride(size_t U) { return (U + kBasisPad - 1) / kBasisPad * kBasisPad; }
+static size_t krylov_v_bytes(size_t U, int cap) { return round256((size_t)(cap + 1) * basis_stride(U) * 8); }
 static size_t krylov_bytes_of(size_t U, int cap, bool fp32) {
   return krylov_v_bytes(U, cap) + round256((size_t)cap * U * (fp32 ? sizeof(float) : sizeof(double)));
 }
@@ -850,9 +852,7 @@ static int setup_impl(const pc_params* p, const double* a_nodes, void* krylov, s
     const size_t U = h->U;
     const int cap = h->cap;
     h->nblocks = num_sms() * kMaxBlocksPerSM;
-    // basis: cap + 1 vectors; a double-float basis stores each as two FP32 planes in
-    // tiles of 512 unknowns (the last tile padded), i.e. ceil(U/512) * 512 doubles per vector
-    const size_t tiled = (U + 511) / 512 * 512;
+    // basis: cap + 1 vectors of whole tiles
     if (krylov) {
       // V and Z in the caller's memory (checked by pc_setup_shared), Z after V
       h->kws = static_cast<const unsigned char*>(krylov);
@@ -860,7 +860,7 @@ static int setup_impl(const pc_params* p, const double* a_nodes, void* krylov, s
       h->V = static_cast<double*>(krylov);
       h->Z = static_cast<unsigned char*>(krylov) + krylov_v_bytes(U, cap);
     } else {
-      if ((rc = dev_alloc_t(h, &h->V, (size_t)(cap + 1) * tiled))) goto fail_out;
+      if ((rc = dev_alloc_t(h, &h->V, (size_t)(cap + 1) * basis_stride(U)))) goto fail_out;
       if ((rc = dev_alloc(h, &h->Z, (size_t)cap * U * (h->fp32 ? sizeof(float) : sizeof(double))))) goto fail_out;
     }
     if (h->fp32 && (rc = dev_alloc_t(h, &h->vf32, U))) goto fail_out;

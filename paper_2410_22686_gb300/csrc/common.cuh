@@ -499,6 +499,11 @@ struct ArnoldiScalars {
   double* flag;  // 1.0 when the step re-orthogonalises
   unsigned* count;  // blocks of a reduction that have finished (zero between launches)
 };
+// The double-float basis (k_krylov.cu) lies in tiles of kBasisTile unknowns, also a streamed
+// stage's (two unknowns a consumer thread); a vector's storage is padded to kBasisPad.
+constexpr int kBasisTile = 256;
+constexpr int kBasisPad = 512;
+static_assert(kBasisPad % kBasisTile == 0, "the padded storage holds whole tiles");
 constexpr int kMaxBlocksPerSM = 8;  // 256-thread blocks: partial-sum buffers hold SMs*8 rows
 // (`prep`: with ww, the reduction also takes the Pythagorean norm; `check`: the update's reduction
 // also decides on re-orthogonalisation)

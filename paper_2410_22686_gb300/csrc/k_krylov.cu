@@ -560,7 +560,7 @@ __global__ void loop_start_kernel(int* jdev, int* kdev, const double* est, doubl
 // (a producer warp issues the bulk asynchronous copies of several stages ahead on
 // mbarriers); the selective second pass reads the hi planes directly.
 // ---------------------------------------------------------------------------
-constexpr int kTile = 256;             // elements per tile of the layout and per streamed stage (two per thread)
+constexpr int kTile = kBasisTile;      // elements per tile of the layout and per streamed stage (two per thread)
 constexpr int kGroup = 16;             // basis vectors per stage of the update
 constexpr int kBarBytes = 256;         // mbarriers (16 full, 16 empty) at the start of the dynamic shared memory
 constexpr int kStreamCtas = 2;         // streaming CTAs an SM
@@ -1208,7 +1208,7 @@ cudaError_t multidot_dispatch(int cnt, Launch& L, const double* V, size_t ldv, i
   }
 }
 
-// one streaming CTA per SM (the stages fill its shared memory), at most one per tile
+// kStreamCtas streaming CTAs per SM (their stages fill its shared memory), at most one per tile
 unsigned stream_grid(size_t len) {
   const size_t ntiles = (len + kTile - 1) / kTile;
   const size_t sms = (size_t)num_sms() * kStreamCtas;
