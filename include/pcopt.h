@@ -510,6 +510,10 @@ int pc_measure_peaks(double* fp64_tflops, double* fp32_tflops, void* stream);
  * usable); PC_ERR_CUDA on a CUDA error.  Allocates nothing.  Synchronises `stream`. */
 int pc_selftest_wait_timeout(double budget_ms, void* stream);
 
+/* Self-test of the FP64 reciprocal of the shifted diagonals (no paper counterpart):
+ * r[i] = 1 / d[i] as the sweeps form it, for n > 0 device values.  Asynchronous on `stream`. */
+int pc_selftest_reciprocal(const double* d, double* r, int64_t n, void* stream);
+
 /* Debug build only (compiled with -DPCOPT_DEBUG, libpcopt_debug.so; no paper
  * counterpart): kernels check their index arithmetic (neighbour indices of the
  * stencils, basis-vector and tile indices of the Krylov kernels, time and column

@@ -101,6 +101,7 @@ _SIGNATURES = {
     "pc_launch_count": (ctypes.c_int64, [_vp]),
     "pc_measure_peaks": (_i, [_dpp, _dpp, _vp]),
     "pc_selftest_wait_timeout": (_i, [_d, _vp]),
+    "pc_selftest_reciprocal": (_i, [_vp, _vp, ctypes.c_int64, _vp]),
     "pc_debug_status": (_i, [_i, _ip]),
     "pc_last_error": (ctypes.c_char_p, []),
     "pc_status_string": (ctypes.c_char_p, [_i]),

@@ -1,4 +1,5 @@
-// Self-tests of the library's failure paths, run on the GPU without faulting it.
+// Self-tests, run on the GPU without faulting it: a failure path, and arithmetic that the
+// solvers use only inside larger sums.
 //
 // pc_selftest_wait_timeout: one CTA announces 64 bytes on an mbarrier and
 // copies only 32 with a bulk asynchronous copy, so the phase can never
@@ -7,6 +8,8 @@
 // by then, so nothing is in flight when the CTA exits.  This is the path the
 // streamed Arnoldi kernels take if a copy ever fails to arrive.  No device
 // memory is allocated: source and error word are file-scope device variables.
+//
+// pc_selftest_reciprocal: rcp_f64 of the values given.
 #include <cuda_runtime.h>
 
 #include <string>
@@ -40,7 +43,21 @@ __global__ void wait_timeout_probe_kernel(const float* src, double* err, long lo
   __syncthreads();
 }
 
+__global__ void reciprocal_kernel(const double* __restrict__ d, double* __restrict__ r, int64_t n) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) r[i] = rcp_f64(d[i]);
+}
+
 }  // namespace
+
+extern "C" int pc_selftest_reciprocal(const double* d, double* r, int64_t n, void* stream) {
+  if (!d || !r || n < 1) return set_error(PC_ERR_ARG, "pc_selftest_reciprocal: null array or n < 1");
+  const int64_t blocks = (n + 255) / 256;
+  reciprocal_kernel<<<(unsigned)(blocks < 1024 ? blocks : 1024), 256, 0, (cudaStream_t)stream>>>(d, r, n);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return set_error(PC_ERR_CUDA, std::string("pc_selftest_reciprocal: ") + cudaGetErrorString(e));
+  return PC_OK;
+}
 
 extern "C" int pc_selftest_wait_timeout(double budget_ms, void* stream) {
   if (!(budget_ms > 0.0) || budget_ms > 10000.0)
