@@ -2455,11 +2455,12 @@ extern "C" int pc_autotune(pc_handle* h, int reps, pc_tiles* chosen, void* strea
       }
     }
   }
-  // the all-at-once matvec of the Arnoldi step: time blocks per thread
+  // the all-at-once matvec of the Arnoldi step: time blocks per thread (every length the rules
+  // by size of k_matvec.cu choose is among them, so a tuned product is not slower than they)
   {
     double tbest = HUGE_VAL;
-    const int tjs[5] = {8, 16, 32, 64, 128};
-    for (int ti = 0; ti < 5; ++ti) {
+    const int tjs[8] = {1, 2, 4, 8, 16, 32, 64, 128};
+    for (int ti = 0; ti < 8; ++ti) {
       if (tjs[ti] > h->n && ti > 0) break;
       Tiles t = best;
       t.mv_tj = tjs[ti];
