@@ -428,12 +428,15 @@ cudaError_t launch_fe3_down(Launch& L, int m, int planes, Tc h, Tc tau, const Tc
       return e;
     // even rows 0, 2, .., m - 1 in strips of 2 cy rows (the last even row needs no strip of its own)
     const unsigned ns = (unsigned)std::max(1, (mc + cy - 1) / cy);
+    const double ev = (double)hm / m, od = (double)mc / m;  // shares of the even and odd layers
     L.begin(KC_MG_SMOOTH);
     fe3_layer_kernel<Tc, 0><<<dim3(ns, (unsigned)hm, (unsigned)planes), kFe3Threads, even, L.stream>>>(r, u, E, sigma,
                                                                                                      m, h, tau, cy);
+    if ((e = L.end(KC_MG_SMOOTH, np * ev * 2.0 * cs, np * ev * 100.0)) != cudaSuccess) return e;
+    L.begin(KC_MG_SMOOTH);
     fe3_layer_kernel<Tc, 1><<<dim3(ns, (unsigned)mc, (unsigned)planes), kFe3Threads, odd, L.stream>>>(r, u, E, sigma, m,
                                                                                                     h, tau, cy);
-    if ((e = L.end(KC_MG_SMOOTH, np * 2.0 * cs, np * 100.0)) != cudaSuccess) return e;
+    if ((e = L.end(KC_MG_SMOOTH, np * od * 2.0 * cs, np * od * 100.0)) != cudaSuccess) return e;
   }
   const int cy = fe3_longest(m, 8, fe3_restrict_smem<Tc>);
   const size_t smem = fe3_restrict_smem<Tc>(m, cy);
