@@ -54,12 +54,15 @@ __device__ __forceinline__ double df_to_f64(const DF& a, int p) {
   return __longlong_as_double((long long)bits);
 }
 
-// Scale 2^p that brings tk into [1, 2): element products keep tk K 2^p in FP32 pairs, so their
-// range is that of K, and take 2^-p in df_to_f64.
+// Scale 2^p that brings tk into [1/2, 1): element products keep tk K 2^p in FP32 pairs, which no
+// K in the FP32 range overflows, and take 2^-p in df_to_f64.
 inline int df_scale_exponent(double tk) {
   int e = 0;
   std::frexp(tk, &e);
-  return 1 - e;
+  return -e;
 }
+// whether the exponent field of df_to_f64's result, Es + 896 - p, holds for every FP32 sum
+// (1 <= Es <= 254); beyond (tau below 1e-270 or above 1e269) the products take FP64 arithmetic
+inline bool df_scale_fits(int p) { return p >= -896 && p <= 896; }
 
 }  // namespace pcopt

@@ -547,13 +547,15 @@ cudaError_t launch_matvec_fevar(Launch& L, int m, int n, double h2, double alpha
   L.begin(KC_MATVEC);
   if constexpr (std::is_same<Tin, float>::value) {
     const int p = df_scale_exponent(tau);
-    if (transpose)
-      fevar_matvec_df_kernel<true><<<grid, 256, 0, L.stream>>>(x, y, E, m, n, tj, h2, alpha, tau, p, xstride, ystride,
-                                                               jdev);
-    else
-      fevar_matvec_df_kernel<false><<<grid, 256, 0, L.stream>>>(x, y, E, m, n, tj, h2, alpha, tau, p, xstride, ystride,
-                                                                jdev);
-    return L.end(KC_MATVEC, tot * (sizeof(Tin) + 8.0), tot * 160.0);
+    if (df_scale_fits(p)) {
+      if (transpose)
+        fevar_matvec_df_kernel<true><<<grid, 256, 0, L.stream>>>(x, y, E, m, n, tj, h2, alpha, tau, p, xstride, ystride,
+                                                                 jdev);
+      else
+        fevar_matvec_df_kernel<false><<<grid, 256, 0, L.stream>>>(x, y, E, m, n, tj, h2, alpha, tau, p, xstride, ystride,
+                                                                  jdev);
+      return L.end(KC_MATVEC, tot * (sizeof(Tin) + 8.0), tot * 160.0);
+    }
   }
   if (transpose)
     fevar_matvec_kernel<Tin, true><<<grid, 256, 0, L.stream>>>(x, y, E, m, n, tj, h2, alpha, tau, xstride, ystride,

@@ -629,22 +629,23 @@ cudaError_t launch_matvec_fevar3(Launch& L, int m, int n, double h, double alpha
   L.begin(KC_MATVEC);
   if constexpr (std::is_same<Tin, float>::value) {
     const int p = df_scale_exponent(tau * kh);
-    if (transpose)
-      fevar3_matvec_df_kernel<true><<<grid, 256, 0, L.stream>>>(x, y, E, m, n, tj, mh, tau * kh, alpha, p, xstride,
-                                                                ystride, jdev);
-    else
-      fevar3_matvec_df_kernel<false><<<grid, 256, 0, L.stream>>>(x, y, E, m, n, tj, mh, tau * kh, alpha, p, xstride,
-                                                                 ystride, jdev);
-    return L.end(KC_MATVEC, tot * (sizeof(Tin) + 8.0), tot * 400.0);
-  } else {
-    if (transpose)
-      fevar3_matvec_kernel<Tin, true><<<grid, 256, 0, L.stream>>>(x, y, E, m, n, tj, mh, kh, alpha, tau, xstride,
+    if (df_scale_fits(p)) {
+      if (transpose)
+        fevar3_matvec_df_kernel<true><<<grid, 256, 0, L.stream>>>(x, y, E, m, n, tj, mh, tau * kh, alpha, p, xstride,
                                                                   ystride, jdev);
-    else
-      fevar3_matvec_kernel<Tin, false><<<grid, 256, 0, L.stream>>>(x, y, E, m, n, tj, mh, kh, alpha, tau, xstride,
+      else
+        fevar3_matvec_df_kernel<false><<<grid, 256, 0, L.stream>>>(x, y, E, m, n, tj, mh, tau * kh, alpha, p, xstride,
                                                                    ystride, jdev);
-    return L.end(KC_MATVEC, tot * (sizeof(Tin) + 8.0), tot * 100.0);
+      return L.end(KC_MATVEC, tot * (sizeof(Tin) + 8.0), tot * 400.0);
+    }
   }
+  if (transpose)
+    fevar3_matvec_kernel<Tin, true><<<grid, 256, 0, L.stream>>>(x, y, E, m, n, tj, mh, kh, alpha, tau, xstride,
+                                                                ystride, jdev);
+  else
+    fevar3_matvec_kernel<Tin, false><<<grid, 256, 0, L.stream>>>(x, y, E, m, n, tj, mh, kh, alpha, tau, xstride,
+                                                                 ystride, jdev);
+  return L.end(KC_MATVEC, tot * (sizeof(Tin) + 8.0), tot * 100.0);
 }
 
 template <typename Tc>
