@@ -1244,16 +1244,14 @@ static cudaError_t spatial_solve(pc_handle* h, Launch& L, int nplanes = 0,
   }
   {
     const CoarseLevels<Tc>& cl = coarse_of<Tc>(h);
-    bool done = false;
-    if constexpr (std::is_same<Tc, float>::value && std::is_same<TU, float2>::value) {
-      if (h->tail2) {
-        if ((e = launch_mg_tail2(L, P, cl, sig, (const C*)h->lv[l0].r, (C*)h->lv[l0].u)) != cudaSuccess) return e;
-        done = true;
-      }
-    }
-    if (!done && (e = launch_mg_coarse_cycle<Tc, TU>(L, h->dim, P, cl, sig, (const C*)h->lv[l0].r,
-                                                     (TU*)h->lv[l0].u)) != cudaSuccess)
-      return e;
+    const C* r0 = (const C*)h->lv[l0].r;
+    TU* u0 = (TU*)h->lv[l0].u;
+    if constexpr (std::is_same<TU, float2>::value)  // in 2D FP32 iterates take the in-place kernel
+      e = h->tail2 ? launch_mg_tail2(L, P, cl, sig, r0, u0) : launch_mg_coarse_cycle<Tc, TU, 3>(L, P, cl, sig, r0, u0);
+    else
+      e = h->dim == 2 ? launch_mg_coarse_cycle<Tc, TU, 2>(L, P, cl, sig, r0, u0)
+                      : launch_mg_coarse_cycle<Tc, TU, 3>(L, P, cl, sig, r0, u0);
+    if (e != cudaSuccess) return e;
   }
   // in 2D the finest level's correction is added by the inverse time transform
   // (fine_correction); in 3D (eight coarse parents per point) by the prolongation kernel
@@ -1307,19 +1305,25 @@ static cudaError_t precond_t(pc_handle* h, Launch& L, const Tin* v, Tout* w, siz
     if (stride != 0 || jdev != nullptr) return cudaErrorNotSupported;  // graph solves reject it first
     return precond_ideal_t<Tc, TU, Tout, Tin>(h, L, v, w);
   }
-  // the chirp-z transforms: host-driven solves only, so no index
-  const ChirpZ<Tc> cz{(const C*)h->cz_tab, h->cz_logM};
-  if (cz.logM && jdev) return cudaErrorNotSupported;
-  cudaError_t e = cz.logM ? launch_tchirp_forward<Tc, Tin>(L, h->ms, h->n, v, Tables<Tc>::dpow(h), cz, (C*)h->lv[0].r)
-                          : launch_tfft_forward<Tc>(L, h->ms, h->n, v, Tables<Tc>::dpow(h), Tables<Tc>::dinv(h),
-                                                    Tables<Tc>::tw(h), (C*)h->lv[0].r,
-                                                    index_input ? (in_stride ? in_stride : stride) : 0,
-                                                    index_input ? jdev : nullptr);
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
+  if constexpr (std::is_same<TU, C>::value) {  // BF16 storage does not take them
+    // the chirp-z transforms: host-driven solves only, so no index
+    const ChirpZ<Tc> cz{(const C*)h->cz_tab, h->cz_logM};
+    if (cz.logM && jdev) return cudaErrorNotSupported;
+    if (cz.logM) {
+      if ((e = launch_tchirp_forward<Tc, Tin>(L, h->ms, h->n, v, Tables<Tc>::dpow(h), cz, (C*)h->lv[0].r)) !=
+          cudaSuccess)
+        return e;
+      if ((e = spatial_solve<Tc, TU>(h, L)) != cudaSuccess) return e;
+      return launch_tchirp_inverse<Tc, Tout>(L, h->ms, h->n, (const C*)h->lv[0].u, Tables<Tc>::dinv(h), cz, w,
+                                             fine_correction<C>(h));
+    }
+  }
+  if ((e = launch_tfft_forward<Tc>(L, h->ms, h->n, v, Tables<Tc>::dpow(h), Tables<Tc>::tw(h), (C*)h->lv[0].r,
+                                   index_input ? (in_stride ? in_stride : stride) : 0,
+                                   index_input ? jdev : nullptr)) != cudaSuccess)
+    return e;
   if ((e = spatial_solve<Tc, TU>(h, L)) != cudaSuccess) return e;
-  if (cz.logM)
-    return launch_tchirp_inverse<Tc, TU, Tout>(L, h->ms, h->n, (const TU*)h->lv[0].u, Tables<Tc>::dinv(h), cz, w,
-                                               fine_correction<TU>(h));
   return launch_tfft_inverse<Tc, TU, Tout>(L, h->ms, h->n, (const TU*)h->lv[0].u, Tables<Tc>::dpow(h),
                                            Tables<Tc>::dinv(h), Tables<Tc>::tw(h), w, stride, jdev,
                                            fine_correction<TU>(h));
@@ -2433,15 +2437,15 @@ extern "C" int pc_autotune(pc_handle* h, int reps, pc_tiles* chosen, void* strea
       const double ms = time_reps(st, reps, [&]() -> cudaError_t {
         typedef float2 C32;
         if (!h->fp32) {
-          cudaError_t e = launch_tfft_forward<double>(L, h->ms, h->n, h->V, h->dpow64, h->dinv64, h->tw64,
+          cudaError_t e = launch_tfft_forward<double>(L, h->ms, h->n, h->V, h->dpow64, h->tw64,
                                                       (double2*)h->lv[0].r);
           if (e != cudaSuccess) return e;
           return launch_tfft_inverse<double, double2, double>(L, h->ms, h->n, (const double2*)h->lv[0].u, h->dpow64,
                                                               h->dinv64, h->tw64, (double*)h->Z);
         }
         // flexible GMRES feeds the FP32 transform with the FP32 copy of the basis vector
-        cudaError_t e = launch_tfft_forward<float>(L, h->ms, h->n, (const float*)h->vf32, h->dpow32, h->dinv32,
-                                                   h->tw32, (C32*)h->lv[0].r);
+        cudaError_t e = launch_tfft_forward<float>(L, h->ms, h->n, (const float*)h->vf32, h->dpow32, h->tw32,
+                                                   (C32*)h->lv[0].r);
         if (e != cudaSuccess) return e;
         if (h->bf16s)
           return launch_tfft_inverse<float, __nv_bfloat162, float>(L, h->ms, h->n, (const __nv_bfloat162*)h->lv[0].u,

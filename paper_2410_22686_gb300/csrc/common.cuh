@@ -351,7 +351,7 @@ cudaError_t launch_fevar3_objective_grad(Launch& L, int m, int n, double h, doub
 // With jdev != nullptr the input is v + (*jdev) * vstride (device-resident Arnoldi index).
 // input v: FP64 basis vectors, or (Tc = float) their FP32 rounding
 template <typename Tc, typename Tin = double>
-cudaError_t launch_tfft_forward(Launch& L, int64_t ms, int n, const Tin* v, const Tc* dpow, const Tc* dinv,
+cudaError_t launch_tfft_forward(Launch& L, int64_t ms, int n, const Tin* v, const Tc* dpow,
                                 const typename Cx<Tc>::t* tw, typename Cx<Tc>::t* spec, size_t vstride = 0,
                                 const int* jdev = nullptr);
 // inverse scaled time FFT + butterfly: spectral planes (stored as TU) -> w (Tout [2][n][ms])
@@ -373,8 +373,8 @@ cudaError_t launch_tfft_inverse(Launch& L, int64_t ms, int n, const TU* spec, co
                                 const int* jdev = nullptr, FineCorrection<TU> fc = FineCorrection<TU>());
 
 // Time transforms of lengths that are not powers of two by the chirp-z method
-// (k_tchirp.cu), n >= kChirpMinN (shorter ones, and FP32 ones around sine-transform solves,
-// take the direct sum of k_tfft.cu).  One
+// (k_tchirp.cu), n >= kChirpMinN (shorter ones, and FP32 ones around sine-transform solves or
+// BF16 storage, take the direct sum of k_tfft.cu).  One
 // table: chirp c_j = exp(-pi i j^2 / n), j < n; filter = DFT_M(conj c) / M at
 // chirp_position; roots exp(-2 pi i q / M), q < M.  logM = 0: no table.
 constexpr int kChirpMinN = 24;
@@ -391,9 +391,9 @@ int chirp_position(int logM, int k);     // where frequency k lies after the for
 template <typename Tc, typename Tin>
 cudaError_t launch_tchirp_forward(Launch& L, int64_t ms, int n, const Tin* v, const Tc* dpow, ChirpZ<Tc> cz,
                                   typename Cx<Tc>::t* spec);
-template <typename Tc, typename TU, typename Tout>
-cudaError_t launch_tchirp_inverse(Launch& L, int64_t ms, int n, const TU* spec, const Tc* dinv, ChirpZ<Tc> cz, Tout* w,
-                                  FineCorrection<TU> fc);
+template <typename Tc, typename Tout>
+cudaError_t launch_tchirp_inverse(Launch& L, int64_t ms, int n, const typename Cx<Tc>::t* spec, const Tc* dinv,
+                                  ChirpZ<Tc> cz, Tout* w, FineCorrection<typename Cx<Tc>::t> fc);
 
 // Sine transforms of any m (k_dst.cu): out = S in along `axis` (S the orthonormal DST-I), or
 // with `divide` out = S diag(rmass / (sigma_p + lamK)) S in (rmass == nullptr: 1).  in may
@@ -483,10 +483,8 @@ constexpr int kMgTailMaxM = 63;
 bool mg_tail2_supported(const CoarseLevels<float>& lv);
 cudaError_t launch_mg_tail2(Launch& L, int planes, const CoarseLevels<float>& lv, const float2* sigma, const float2* r0,
                             float2* u0);
-template <typename Tc, typename TU>
-size_t mg_coarse_cycle_smem(const CoarseLevels<Tc>& lv);
-template <typename Tc, typename TU>
-cudaError_t launch_mg_coarse_cycle(Launch& L, int dim, int planes, const CoarseLevels<Tc>& lv,
+template <typename Tc, typename TU, int DIM>
+cudaError_t launch_mg_coarse_cycle(Launch& L, int planes, const CoarseLevels<Tc>& lv,
                                    const typename Cx<Tc>::t* sigma, const typename Cx<Tc>::t* r0, TU* u0);
 
 // Krylov (FP64).  Device scalars of one Arnoldi step.

@@ -863,7 +863,7 @@ __global__ void __launch_bounds__(1024) mg_coarse_cycle_kernel(const CoarseLevel
 }  // namespace
 
 template <typename Tc, typename TU>
-size_t mg_coarse_cycle_smem(const CoarseLevels<Tc>& lv) {
+static size_t mg_coarse_cycle_smem(const CoarseLevels<Tc>& lv) {
   size_t b = 0;
   for (int l = 0; l < lv.count; ++l)
     b += 2 * (size_t)lv.np[l] * sizeof(typename Cx<Tc>::t) + (((size_t)lv.np[l] * sizeof(TU) + 15) / 16) * 16;
@@ -878,38 +878,33 @@ static size_t coarse_coef_smem(const CoarseLevels<Tc>& lv, int dim) {
   return b;
 }
 
-template <typename Tc, typename TU>
-cudaError_t launch_mg_coarse_cycle(Launch& L, int dim, int planes, const CoarseLevels<Tc>& lv,
+template <typename Tc, typename TU, int DIM>
+cudaError_t launch_mg_coarse_cycle(Launch& L, int planes, const CoarseLevels<Tc>& lv,
                                    const typename Cx<Tc>::t* sigma, const typename Cx<Tc>::t* r0, TU* u0) {
   // stage the coefficients too when everything fits beside the levels
   const size_t base = mg_coarse_cycle_smem<Tc, TU>(lv);
-  const size_t coef = coarse_coef_smem<Tc>(lv, dim);
+  const size_t coef = coarse_coef_smem<Tc>(lv, DIM);
   const int stage = base + coef <= 200 * 1024 ? 1 : 0;
   const size_t smem = base + (stage ? coef : 0);
-  cudaError_t e;
-  if (dim == 2)
-    e = allow_dynamic_smem(mg_coarse_cycle_kernel<Tc, TU, 2>, smem);
-  else
-    e = allow_dynamic_smem(mg_coarse_cycle_kernel<Tc, TU, 3>, smem);
+  cudaError_t e = allow_dynamic_smem(mg_coarse_cycle_kernel<Tc, TU, DIM>, smem);
   if (e != cudaSuccess) return e;
   double pts = 0;
   for (int l = 0; l < lv.count; ++l) pts += (double)lv.np[l];
   const double cs = sizeof(typename Cx<Tc>::t);
   L.begin(KC_MG_COARSE);
-  if (dim == 2)
-    mg_coarse_cycle_kernel<Tc, TU, 2><<<planes, coarse_threads<Tc>(), smem, L.stream>>>(lv, r0, u0, sigma, stage);
-  else
-    mg_coarse_cycle_kernel<Tc, TU, 3><<<planes, coarse_threads<Tc>(), smem, L.stream>>>(lv, r0, u0, sigma, stage);
+  mg_coarse_cycle_kernel<Tc, TU, DIM><<<planes, coarse_threads<Tc>(), smem, L.stream>>>(lv, r0, u0, sigma, stage);
   return L.end(KC_MG_COARSE, (double)planes * lv.np[0] * (cs + sizeof(TU)), (double)planes * pts * 60.0);
 }
 
-#define PCOPT_INST_CC(Tc, TU)                                                                              \
-  template cudaError_t launch_mg_coarse_cycle<Tc, TU>(Launch&, int, int, const CoarseLevels<Tc>&,         \
-                                                      const Cx<Tc>::t*, const Cx<Tc>::t*, TU*);            \
-  template size_t mg_coarse_cycle_smem<Tc, TU>(const CoarseLevels<Tc>&);
-PCOPT_INST_CC(float, float2)
-PCOPT_INST_CC(double, double2)
-PCOPT_INST_CC(float, __nv_bfloat162)
+// (2D with FP32 iterates: k_mgtail.cu)
+#define PCOPT_INST_CC(Tc, TU, DIM)                                                           \
+  template cudaError_t launch_mg_coarse_cycle<Tc, TU, DIM>(Launch&, int, const CoarseLevels<Tc>&, \
+                                                           const Cx<Tc>::t*, const Cx<Tc>::t*, TU*);
+PCOPT_INST_CC(float, float2, 3)
+PCOPT_INST_CC(double, double2, 2)
+PCOPT_INST_CC(double, double2, 3)
+PCOPT_INST_CC(float, __nv_bfloat162, 2)
+PCOPT_INST_CC(float, __nv_bfloat162, 3)
 #undef PCOPT_INST_CC
 
 }  // namespace pcopt

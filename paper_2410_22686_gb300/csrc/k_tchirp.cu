@@ -20,10 +20,11 @@
 // 53.5 -> 17.2 us, n = 31 71.9 -> 16.8, n = 100 343 -> 39, n = 511 2058 -> 162;
 // FP32: n = 24 12.6 -> 7.8, n = 100 77.9 -> 10.6, n = 511 391 -> 19.
 //
-// FP32 transforms around sine-transform solves keep the direct sum at every length: what such
-// a solve leaves at rtol is FP32 rounding amplified by A, and another order of the sums moves
-// its solution by up to rtol (31^2 x 63 at rtol = 1e-8: 9.5e-9).  Around multigrid the cycle's
-// own error is what is left there, and the solutions agree to 1e-12.
+// FP32 transforms around sine-transform solves and BF16 storage keep the direct sum at every
+// length: what such a solve leaves at rtol is FP32 rounding amplified by A (or flipped BF16
+// roundings), and another order of the sums moves its solution by up to rtol (31^2 x 63 at rtol =
+// 1e-8: 9.5e-9).  Around multigrid with FP32 storage the cycle's own error is what is left
+// there, and the solutions agree to 1e-12.
 #include <algorithm>
 
 #include "common.cuh"
@@ -212,11 +213,11 @@ __global__ void __launch_bounds__(kCzThreads, 2) tchirp_forward_kernel(const Tin
 
 // The inverse transform is the forward one with real and imaginary parts exchanged on
 // both sides.
-template <typename Tc, typename TU, typename Tout>
-__global__ void __launch_bounds__(kCzThreads, 2) tchirp_inverse_kernel(const TU* __restrict__ spec,
+template <typename Tc, typename Tout>
+__global__ void __launch_bounds__(kCzThreads, 2) tchirp_inverse_kernel(const typename Cx<Tc>::t* __restrict__ spec,
                                                                        const Tc* __restrict__ dinv, ChirpZ<Tc> cz,
                                                                        Tout* __restrict__ w, int64_t ms, int n, int lc,
-                                                                       FineCorrection<TU> fc) {
+                                                                       FineCorrection<typename Cx<Tc>::t> fc) {
   typedef typename Cx<Tc>::t C;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const CzTile<Tc> t{reinterpret_cast<C*>(smem_raw), cz.roots(n), 1 << cz.logM, lc};
@@ -227,10 +228,10 @@ __global__ void __launch_bounds__(kCzThreads, 2) tchirp_inverse_kernel(const TU*
     const int64_t s = s0 + c;
     C sa = czero<Tc>(), sb = czero<Tc>();
     if (s < ms) {
-      sa = ldc(spec, (int64_t)(2 * k) * ms + s);
-      sb = ldc(spec, (int64_t)(2 * k + 1) * ms + s);
+      sa = spec[(int64_t)(2 * k) * ms + s];
+      sb = spec[(int64_t)(2 * k + 1) * ms + s];
       if (fc.ec) {
-        Parents<Tc, TU> par;
+        Parents<Tc, C> par;
         par.init(fc, s);
         sa = par.corrected(sa, fc, 2 * k);
         sb = par.corrected(sb, fc, 2 * k + 1);
@@ -302,19 +303,19 @@ cudaError_t launch_tchirp_forward(Launch& L, int64_t ms, int n, const Tin* v, co
                (double)ms * (10.0 * cz.logM + 6.0) * (1 << cz.logM));
 }
 
-template <typename Tc, typename TU, typename Tout>
-cudaError_t launch_tchirp_inverse(Launch& L, int64_t ms, int n, const TU* spec, const Tc* dinv, ChirpZ<Tc> cz, Tout* w,
-                                  FineCorrection<TU> fc) {
+template <typename Tc, typename Tout>
+cudaError_t launch_tchirp_inverse(Launch& L, int64_t ms, int n, const typename Cx<Tc>::t* spec, const Tc* dinv,
+                                  ChirpZ<Tc> cz, Tout* w, FineCorrection<typename Cx<Tc>::t> fc) {
   typedef typename Cx<Tc>::t C;
   const int lc = cz_lc<Tc>(cz.logM, ms);
   const size_t smem = sizeof(C) << (cz.logM + lc);
-  auto kern = tchirp_inverse_kernel<Tc, TU, Tout>;
+  auto kern = tchirp_inverse_kernel<Tc, Tout>;
   cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
-  const double cbytes = fc.ec ? (double)(n / 2 + 1) * 2.0 * fc.npc * sizeof(TU) : 0.0;
+  const double cbytes = fc.ec ? (double)(n / 2 + 1) * 2.0 * fc.npc * sizeof(C) : 0.0;
   L.begin(KC_TFFT_INV);
   kern<<<(unsigned)((ms + (1 << lc) - 1) >> lc), kCzThreads, smem, L.stream>>>(spec, dinv, cz, w, ms, n, lc, fc);
-  return L.end(KC_TFFT_INV, 2.0 * (n / 2 + 1) * ms * sizeof(TU) + 2.0 * n * ms * sizeof(Tout) + cbytes,
+  return L.end(KC_TFFT_INV, 2.0 * (n / 2 + 1) * ms * sizeof(C) + 2.0 * n * ms * sizeof(Tout) + cbytes,
                (double)ms * (10.0 * cz.logM + 6.0) * (1 << cz.logM));
 }
 
@@ -324,14 +325,12 @@ template cudaError_t launch_tchirp_forward<float, double>(Launch&, int64_t, int,
                                                           ChirpZ<float>, float2*);
 template cudaError_t launch_tchirp_forward<float, float>(Launch&, int64_t, int, const float*, const float*,
                                                          ChirpZ<float>, float2*);
-#define PCOPT_INV(Tc, TU, Tout)                                                                                   \
-  template cudaError_t launch_tchirp_inverse<Tc, TU, Tout>(Launch&, int64_t, int, const TU*, const Tc*, ChirpZ<Tc>, \
-                                                           Tout*, FineCorrection<TU>);
-PCOPT_INV(double, double2, double)
-PCOPT_INV(float, float2, double)
-PCOPT_INV(float, float2, float)
-PCOPT_INV(float, __nv_bfloat162, double)
-PCOPT_INV(float, __nv_bfloat162, float)
+#define PCOPT_INV(Tc, Tout)                                                                                       \
+  template cudaError_t launch_tchirp_inverse<Tc, Tout>(Launch&, int64_t, int, const Cx<Tc>::t*, const Tc*, ChirpZ<Tc>, \
+                                                       Tout*, FineCorrection<Cx<Tc>::t>);
+PCOPT_INV(double, double)
+PCOPT_INV(float, double)
+PCOPT_INV(float, float)
 #undef PCOPT_INV
 
 }  // namespace pcopt

@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(256) tfft_inverse_kernel(const TU* __restrict_
 // v1[n-1-j] and v2[j] of the thread's column (zero outside the grid).  Returns after
 // the spectrum stores; the caller's barrier orders the reuse of `sm`.
 template <typename Tc, int N1, int N2, int NT, typename Ld>
-__device__ __forceinline__ void fwd4_body(Ld&& ld, const Tc* __restrict__ dpow, const Tc* __restrict__ dinv,
+__device__ __forceinline__ void fwd4_body(Ld&& ld, const Tc* __restrict__ dpow,
                                           const typename Cx<Tc>::t* __restrict__ tw,
                                           typename Cx<Tc>::t* __restrict__ spec, typename Cx<Tc>::t* sm,
                                           int64_t ms, int64_t s, bool valid, int r, int c) {
@@ -226,7 +226,7 @@ __device__ __forceinline__ void fwd4_body(Ld&& ld, const Tc* __restrict__ dpow, 
 // ld(k, sa, sb) gives spectral planes 2k and 2k+1 of the thread's column (zero
 // outside the grid).  Returns after the output stores.
 template <typename Tc, typename Tout, int N1, int N2, int NT, typename Ld>
-__device__ __forceinline__ void inv4_body(Ld&& ld, const Tc* __restrict__ dpow, const Tc* __restrict__ dinv,
+__device__ __forceinline__ void inv4_body(Ld&& ld, const Tc* __restrict__ dinv,
                                           const typename Cx<Tc>::t* __restrict__ tw, Tout* __restrict__ w,
                                           typename Cx<Tc>::t* sm, int64_t ms, int64_t s, bool valid, int r,
                                           int c) {
@@ -304,7 +304,6 @@ constexpr int tfft_fp64_blocks() {
 // one CTA per tile, inputs loaded straight into registers
 template <typename Tin, typename Tc, int N1, int N2, int NT>
 __global__ void __launch_bounds__(NT) tfft4_forward_kernel(const Tin* __restrict__ v, const Tc* __restrict__ dpow,
-                                                            const Tc* __restrict__ dinv,
                                                             const typename Cx<Tc>::t* __restrict__ tw,
                                                             typename Cx<Tc>::t* __restrict__ spec, int64_t ms,
                                                             size_t vstride, const int* __restrict__ jdev) {
@@ -325,7 +324,7 @@ __global__ void __launch_bounds__(NT) tfft4_forward_kernel(const Tin* __restrict
         a = valid ? cvt<Tc>(v1[(int64_t)(n - 1 - j) * ms + s]) : Tc(0);
         b = valid ? cvt<Tc>(v2[(int64_t)j * ms + s]) : Tc(0);
       },
-      dpow, dinv, tw, spec, sm, ms, s, valid, r, c);
+      dpow, tw, spec, sm, ms, s, valid, r, c);
 }
 
 // the same for FP64 transforms of up to 256 points, compiled for two CTAs per SM
@@ -333,7 +332,6 @@ __global__ void __launch_bounds__(NT) tfft4_forward_kernel(const Tin* __restrict
 template <typename Tin, int N1, int N2, int NT>
 __global__ void __launch_bounds__(NT, 512 / NT) tfft4_forward_f64_kernel(const Tin* __restrict__ v,
                                                                    const double* __restrict__ dpow,
-                                                                   const double* __restrict__ dinv,
                                                                    const double2* __restrict__ tw,
                                                                    double2* __restrict__ spec, int64_t ms,
                                                                    size_t vstride, const int* __restrict__ jdev) {
@@ -353,7 +351,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) tfft4_forward_f64_kernel(const T
         a = valid ? cvt<double>(v1[(int64_t)(n - 1 - j) * ms + s]) : 0.0;
         b = valid ? cvt<double>(v2[(int64_t)j * ms + s]) : 0.0;
       },
-      dpow, dinv, tw, spec, sm, ms, s, valid, r, c);
+      dpow, tw, spec, sm, ms, s, valid, r, c);
 }
 
 // Persistent streaming variant: each CTA walks tiles blockIdx.x, + gridDim.x, ...
@@ -361,7 +359,6 @@ __global__ void __launch_bounds__(NT, 512 / NT) tfft4_forward_f64_kernel(const T
 // with cp.async while it transforms the current one.
 template <typename Tin, typename Tc, int N1, int N2>
 __global__ void __launch_bounds__(256) tfft4s_forward_kernel(const Tin* __restrict__ v, const Tc* __restrict__ dpow,
-                                                             const Tc* __restrict__ dinv,
                                                              const typename Cx<Tc>::t* __restrict__ tw,
                                                              typename Cx<Tc>::t* __restrict__ spec, int64_t ms,
                                                              int ntiles, size_t vstride, const int* __restrict__ jdev) {
@@ -402,15 +399,14 @@ __global__ void __launch_bounds__(256) tfft4s_forward_kernel(const Tin* __restri
           a = cvt<Tc>(st[(n - 1 - j) * COLS + c]);
           b = cvt<Tc>(st[(n + j) * COLS + c]);
         },
-        dpow, dinv, tw, spec, sm, ms, s, s < ms, r, c);
+        dpow, tw, spec, sm, ms, s, s < ms, r, c);
     __syncthreads();  // stage[buf] and sm are rewritten next
   }
   cp_async_wait<0>();
 }
 
 template <typename Tc, typename TU, typename Tout, int N1, int N2, int NT>
-__global__ void __launch_bounds__(NT, ((sizeof(Tc) == 4 && N1 * N2 <= 256) ? 4 : tfft_fp64_blocks<Tc, N1 * N2>()) * (256 / NT)) tfft4_inverse_kernel(const TU* __restrict__ spec, const Tc* __restrict__ dpow,
-                                                            const Tc* __restrict__ dinv,
+__global__ void __launch_bounds__(NT, ((sizeof(Tc) == 4 && N1 * N2 <= 256) ? 4 : tfft_fp64_blocks<Tc, N1 * N2>()) * (256 / NT)) tfft4_inverse_kernel(const TU* __restrict__ spec, const Tc* __restrict__ dinv,
                                                             const typename Cx<Tc>::t* __restrict__ tw,
                                                             Tout* __restrict__ w, int64_t ms, size_t wstride,
                                                             const int* __restrict__ jdev, FineCorrection<TU> fc) {
@@ -438,14 +434,13 @@ __global__ void __launch_bounds__(NT, ((sizeof(Tc) == 4 && N1 * N2 <= 256) ? 4 :
           }
         }
       },
-      dpow, dinv, tw, w, sm, ms, s, valid, r, c);
+      dinv, tw, w, sm, ms, s, valid, r, c);
 }
 
 // Persistent streaming inverse: the next tile's 2 (n/2 + 1) spectral planes are
 // copied into a second stage with cp.async while the current tile is transformed.
 template <typename Tc, typename TU, typename Tout, int N1, int N2>
-__global__ void __launch_bounds__(256) tfft4s_inverse_kernel(const TU* __restrict__ spec, const Tc* __restrict__ dpow,
-                                                             const Tc* __restrict__ dinv,
+__global__ void __launch_bounds__(256) tfft4s_inverse_kernel(const TU* __restrict__ spec, const Tc* __restrict__ dinv,
                                                              const typename Cx<Tc>::t* __restrict__ tw,
                                                              Tout* __restrict__ w, int64_t ms, int ntiles,
                                                              size_t wstride, const int* __restrict__ jdev,
@@ -495,7 +490,7 @@ __global__ void __launch_bounds__(256) tfft4s_inverse_kernel(const TU* __restric
             sb = par.corrected(sb, fc, 2 * k + 1);
           }
         },
-        dpow, dinv, tw, w, sm, ms, s, valid, r, c);
+        dinv, tw, w, sm, ms, s, valid, r, c);
     __syncthreads();
   }
   cp_async_wait<0>();
@@ -508,7 +503,6 @@ __global__ void __launch_bounds__(256) tfft4s_inverse_kernel(const TU* __restric
 // sum with the twiddle index advanced incrementally modulo n.  n^2 work per column.
 template <typename Tc, typename Tin>
 __global__ void __launch_bounds__(256) tdft_forward_kernel(const Tin* __restrict__ v, const Tc* __restrict__ dpow,
-                                                           const Tc* __restrict__ dinv,
                                                            const typename Cx<Tc>::t* __restrict__ tw,
                                                            typename Cx<Tc>::t* __restrict__ spec, int64_t ms, int n,
                                                            int TS) {
@@ -555,8 +549,7 @@ __global__ void __launch_bounds__(256) tdft_forward_kernel(const Tin* __restrict
 }
 
 template <typename Tc, typename TU, typename Tout>
-__global__ void __launch_bounds__(256) tdft_inverse_kernel(const TU* __restrict__ spec, const Tc* __restrict__ dpow,
-                                                           const Tc* __restrict__ dinv,
+__global__ void __launch_bounds__(256) tdft_inverse_kernel(const TU* __restrict__ spec, const Tc* __restrict__ dinv,
                                                            const typename Cx<Tc>::t* __restrict__ tw,
                                                            Tout* __restrict__ w, int64_t ms, int n, int TS,
                                                            FineCorrection<TU> fc) {
@@ -646,7 +639,7 @@ int ilog2(int n) {
 static bool small_tiles(int64_t ms, int cols) { return (ms + cols - 1) / cols < 2 * num_sms(); }
 
 template <typename Tin, typename Tc, int N1, int N2, int NT>
-cudaError_t fwd4_nt(Launch& L, int64_t ms, const Tin* v, const Tc* dpow, const Tc* dinv, const typename Cx<Tc>::t* tw,
+cudaError_t fwd4_nt(Launch& L, int64_t ms, const Tin* v, const Tc* dpow, const typename Cx<Tc>::t* tw,
                     typename Cx<Tc>::t* spec, size_t vstride, const int* jdev) {
   constexpr int COLS = NT / N1;
   const size_t smem = (size_t)N1 * N2 * COLS * sizeof(typename Cx<Tc>::t);
@@ -655,26 +648,26 @@ cudaError_t fwd4_nt(Launch& L, int64_t ms, const Tin* v, const Tc* dpow, const T
     auto kern = tfft4_forward_f64_kernel<Tin, N1, N2, NT>;
     cudaError_t e = allow_dynamic_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    kern<<<blocks, NT, smem, L.stream>>>(v, dpow, dinv, tw, spec, ms, vstride, jdev);
+    kern<<<blocks, NT, smem, L.stream>>>(v, dpow, tw, spec, ms, vstride, jdev);
   } else {
     auto kern = tfft4_forward_kernel<Tin, Tc, N1, N2, NT>;
     cudaError_t e = allow_dynamic_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    kern<<<blocks, NT, smem, L.stream>>>(v, dpow, dinv, tw, spec, ms, vstride, jdev);
+    kern<<<blocks, NT, smem, L.stream>>>(v, dpow, tw, spec, ms, vstride, jdev);
   }
   return cudaGetLastError();
 }
 
 template <typename Tin, typename Tc, int N1, int N2>
-cudaError_t fwd4(Launch& L, int64_t ms, const Tin* v, const Tc* dpow, const Tc* dinv, const typename Cx<Tc>::t* tw,
+cudaError_t fwd4(Launch& L, int64_t ms, const Tin* v, const Tc* dpow, const typename Cx<Tc>::t* tw,
                  typename Cx<Tc>::t* spec, size_t vstride, const int* jdev) {
   if constexpr (N1 >= 4 && N1 <= 16)
-    if (small_tiles(ms, 256 / N1)) return fwd4_nt<Tin, Tc, N1, N2, 64>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev);
-  return fwd4_nt<Tin, Tc, N1, N2, 256>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev);
+    if (small_tiles(ms, 256 / N1)) return fwd4_nt<Tin, Tc, N1, N2, 64>(L, ms, v, dpow, tw, spec, vstride, jdev);
+  return fwd4_nt<Tin, Tc, N1, N2, 256>(L, ms, v, dpow, tw, spec, vstride, jdev);
 }
 
 template <typename Tc, typename TU, typename Tout, int N1, int N2, int NT>
-cudaError_t inv4_nt(Launch& L, int64_t ms, const TU* spec, const Tc* dpow, const Tc* dinv,
+cudaError_t inv4_nt(Launch& L, int64_t ms, const TU* spec, const Tc* dinv,
                     const typename Cx<Tc>::t* tw, Tout* w, size_t wstride, const int* jdev,
                     const FineCorrection<TU>& fc) {
   constexpr int COLS = NT / N1;
@@ -682,28 +675,28 @@ cudaError_t inv4_nt(Launch& L, int64_t ms, const TU* spec, const Tc* dpow, const
   auto kern = tfft4_inverse_kernel<Tc, TU, Tout, N1, N2, NT>;
   cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)((ms + COLS - 1) / COLS), NT, smem, L.stream>>>(spec, dpow, dinv, tw, w, ms, wstride, jdev, fc);
+  kern<<<(unsigned)((ms + COLS - 1) / COLS), NT, smem, L.stream>>>(spec, dinv, tw, w, ms, wstride, jdev, fc);
   return cudaGetLastError();
 }
 
 template <typename Tc, typename TU, typename Tout, int N1, int N2>
-cudaError_t inv4(Launch& L, int64_t ms, const TU* spec, const Tc* dpow, const Tc* dinv, const typename Cx<Tc>::t* tw,
+cudaError_t inv4(Launch& L, int64_t ms, const TU* spec, const Tc* dinv, const typename Cx<Tc>::t* tw,
                  Tout* w, size_t wstride, const int* jdev, const FineCorrection<TU>& fc) {
   if constexpr (N1 >= 4 && N1 <= 16)
     if (small_tiles(ms, 256 / N1))
-      return inv4_nt<Tc, TU, Tout, N1, N2, 64>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc);
-  return inv4_nt<Tc, TU, Tout, N1, N2, 256>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc);
+      return inv4_nt<Tc, TU, Tout, N1, N2, 64>(L, ms, spec, dinv, tw, w, wstride, jdev, fc);
+  return inv4_nt<Tc, TU, Tout, N1, N2, 256>(L, ms, spec, dinv, tw, w, wstride, jdev, fc);
 }
 
 static int sm_count(const Launch& L) { return L.tiles && L.tiles->sms > 0 ? L.tiles->sms : 152; }
 
 template <typename Tin, typename Tc, int N1, int N2>
-cudaError_t fwd4s(Launch& L, int64_t ms, const Tin* v, const Tc* dpow, const Tc* dinv,
+cudaError_t fwd4s(Launch& L, int64_t ms, const Tin* v, const Tc* dpow,
                   const typename Cx<Tc>::t* tw, typename Cx<Tc>::t* spec, size_t vstride, const int* jdev) {
   constexpr int n = N1 * N2;
   constexpr int COLS = 256 / N1;
   const size_t smem = (size_t)2 * 2 * n * COLS * sizeof(Tin) + (size_t)n * COLS * sizeof(typename Cx<Tc>::t);
-  if (smem > 227 * 1024) return fwd4<Tin, Tc, N1, N2>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev);
+  if (smem > 227 * 1024) return fwd4<Tin, Tc, N1, N2>(L, ms, v, dpow, tw, spec, vstride, jdev);
   auto kern = tfft4s_forward_kernel<Tin, Tc, N1, N2>;
   cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
@@ -711,12 +704,12 @@ cudaError_t fwd4s(Launch& L, int64_t ms, const Tin* v, const Tc* dpow, const Tc*
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem)) != cudaSuccess) return e;
   const int ntiles = (int)((ms + COLS - 1) / COLS);
   const int grid = std::min(ntiles, std::max(1, per_sm) * sm_count(L));
-  kern<<<grid, 256, smem, L.stream>>>(v, dpow, dinv, tw, spec, ms, ntiles, vstride, jdev);
+  kern<<<grid, 256, smem, L.stream>>>(v, dpow, tw, spec, ms, ntiles, vstride, jdev);
   return cudaGetLastError();
 }
 
 template <typename Tc, typename TU, typename Tout, int N1, int N2>
-cudaError_t inv4s(Launch& L, int64_t ms, const TU* spec, const Tc* dpow, const Tc* dinv,
+cudaError_t inv4s(Launch& L, int64_t ms, const TU* spec, const Tc* dinv,
                   const typename Cx<Tc>::t* tw, Tout* w, size_t wstride, const int* jdev,
                   const FineCorrection<TU>& fc) {
   constexpr int n = N1 * N2;
@@ -724,7 +717,7 @@ cudaError_t inv4s(Launch& L, int64_t ms, const TU* spec, const Tc* dpow, const T
   constexpr int NP = 2 * (n / 2 + 1);
   const size_t smem = (((size_t)2 * NP * COLS * sizeof(TU) + 15) / 16) * 16 +
                       (size_t)n * COLS * sizeof(typename Cx<Tc>::t);
-  if (smem > 227 * 1024) return inv4<Tc, TU, Tout, N1, N2>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc);
+  if (smem > 227 * 1024) return inv4<Tc, TU, Tout, N1, N2>(L, ms, spec, dinv, tw, w, wstride, jdev, fc);
   auto kern = tfft4s_inverse_kernel<Tc, TU, Tout, N1, N2>;
   cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
@@ -732,7 +725,7 @@ cudaError_t inv4s(Launch& L, int64_t ms, const TU* spec, const Tc* dpow, const T
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem)) != cudaSuccess) return e;
   const int ntiles = (int)((ms + COLS - 1) / COLS);
   const int grid = std::min(ntiles, std::max(1, per_sm) * sm_count(L));
-  kern<<<grid, 256, smem, L.stream>>>(spec, dpow, dinv, tw, w, ms, ntiles, wstride, jdev, fc);
+  kern<<<grid, 256, smem, L.stream>>>(spec, dinv, tw, w, ms, ntiles, wstride, jdev, fc);
   return cudaGetLastError();
 }
 
@@ -743,78 +736,78 @@ constexpr int four_step_max() {
 }
 
 template <typename Tin, typename Tc>
-cudaError_t fwd4_dispatch(Launch& L, int64_t ms, int n, const Tin* v, const Tc* dpow, const Tc* dinv,
+cudaError_t fwd4_dispatch(Launch& L, int64_t ms, int n, const Tin* v, const Tc* dpow,
                           const typename Cx<Tc>::t* tw, typename Cx<Tc>::t* spec, size_t vstride, const int* jdev) {
   const bool stream = L.tiles && L.tiles->fft_stream > 0;
   switch (n) {
-    case 1: return stream ? fwd4s<Tin, Tc, 1, 1>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev)
-                    : fwd4<Tin, Tc, 1, 1>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev);
-    case 2: return stream ? fwd4s<Tin, Tc, 2, 1>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev)
-                    : fwd4<Tin, Tc, 2, 1>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev);
-    case 4: return stream ? fwd4s<Tin, Tc, 2, 2>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev)
-                    : fwd4<Tin, Tc, 2, 2>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev);
-    case 8: return stream ? fwd4s<Tin, Tc, 4, 2>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev)
-                    : fwd4<Tin, Tc, 4, 2>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev);
-    case 16: return stream ? fwd4s<Tin, Tc, 4, 4>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev)
-                    : fwd4<Tin, Tc, 4, 4>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev);
-    case 32: return stream ? fwd4s<Tin, Tc, 8, 4>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev)
-                    : fwd4<Tin, Tc, 8, 4>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev);
-    case 64: return stream ? fwd4s<Tin, Tc, 8, 8>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev)
-                    : fwd4<Tin, Tc, 8, 8>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev);
-    case 128: return stream ? fwd4s<Tin, Tc, 16, 8>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev)
-                    : fwd4<Tin, Tc, 16, 8>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev);
-    case 256: return stream ? fwd4s<Tin, Tc, 16, 16>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev)
-                    : fwd4<Tin, Tc, 16, 16>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev);
+    case 1: return stream ? fwd4s<Tin, Tc, 1, 1>(L, ms, v, dpow, tw, spec, vstride, jdev)
+                    : fwd4<Tin, Tc, 1, 1>(L, ms, v, dpow, tw, spec, vstride, jdev);
+    case 2: return stream ? fwd4s<Tin, Tc, 2, 1>(L, ms, v, dpow, tw, spec, vstride, jdev)
+                    : fwd4<Tin, Tc, 2, 1>(L, ms, v, dpow, tw, spec, vstride, jdev);
+    case 4: return stream ? fwd4s<Tin, Tc, 2, 2>(L, ms, v, dpow, tw, spec, vstride, jdev)
+                    : fwd4<Tin, Tc, 2, 2>(L, ms, v, dpow, tw, spec, vstride, jdev);
+    case 8: return stream ? fwd4s<Tin, Tc, 4, 2>(L, ms, v, dpow, tw, spec, vstride, jdev)
+                    : fwd4<Tin, Tc, 4, 2>(L, ms, v, dpow, tw, spec, vstride, jdev);
+    case 16: return stream ? fwd4s<Tin, Tc, 4, 4>(L, ms, v, dpow, tw, spec, vstride, jdev)
+                    : fwd4<Tin, Tc, 4, 4>(L, ms, v, dpow, tw, spec, vstride, jdev);
+    case 32: return stream ? fwd4s<Tin, Tc, 8, 4>(L, ms, v, dpow, tw, spec, vstride, jdev)
+                    : fwd4<Tin, Tc, 8, 4>(L, ms, v, dpow, tw, spec, vstride, jdev);
+    case 64: return stream ? fwd4s<Tin, Tc, 8, 8>(L, ms, v, dpow, tw, spec, vstride, jdev)
+                    : fwd4<Tin, Tc, 8, 8>(L, ms, v, dpow, tw, spec, vstride, jdev);
+    case 128: return stream ? fwd4s<Tin, Tc, 16, 8>(L, ms, v, dpow, tw, spec, vstride, jdev)
+                    : fwd4<Tin, Tc, 16, 8>(L, ms, v, dpow, tw, spec, vstride, jdev);
+    case 256: return stream ? fwd4s<Tin, Tc, 16, 16>(L, ms, v, dpow, tw, spec, vstride, jdev)
+                    : fwd4<Tin, Tc, 16, 16>(L, ms, v, dpow, tw, spec, vstride, jdev);
     case 512:
-      if constexpr (sizeof(Tc) == 4) return stream ? fwd4s<Tin, Tc, 32, 16>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev)
-                    : fwd4<Tin, Tc, 32, 16>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev);
+      if constexpr (sizeof(Tc) == 4) return stream ? fwd4s<Tin, Tc, 32, 16>(L, ms, v, dpow, tw, spec, vstride, jdev)
+                    : fwd4<Tin, Tc, 32, 16>(L, ms, v, dpow, tw, spec, vstride, jdev);
       break;
     case 1024:
-      if constexpr (sizeof(Tc) == 4) return stream ? fwd4s<Tin, Tc, 32, 32>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev)
-                    : fwd4<Tin, Tc, 32, 32>(L, ms, v, dpow, dinv, tw, spec, vstride, jdev);
+      if constexpr (sizeof(Tc) == 4) return stream ? fwd4s<Tin, Tc, 32, 32>(L, ms, v, dpow, tw, spec, vstride, jdev)
+                    : fwd4<Tin, Tc, 32, 32>(L, ms, v, dpow, tw, spec, vstride, jdev);
       break;
   }
   return cudaErrorInvalidValue;
 }
 
 template <typename Tc, typename TU, typename Tout>
-cudaError_t inv4_dispatch(Launch& L, int64_t ms, int n, const TU* spec, const Tc* dpow, const Tc* dinv,
+cudaError_t inv4_dispatch(Launch& L, int64_t ms, int n, const TU* spec, const Tc* dinv,
                           const typename Cx<Tc>::t* tw, Tout* w, size_t wstride, const int* jdev,
                           const FineCorrection<TU>& fc) {
   const bool stream = L.tiles && L.tiles->fft_stream > 0;
   switch (n) {
-    case 1: return stream ? inv4s<Tc, TU, Tout, 1, 1>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc)
-                    : inv4<Tc, TU, Tout, 1, 1>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc);
-    case 2: return stream ? inv4s<Tc, TU, Tout, 2, 1>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc)
-                    : inv4<Tc, TU, Tout, 2, 1>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc);
-    case 4: return stream ? inv4s<Tc, TU, Tout, 2, 2>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc)
-                    : inv4<Tc, TU, Tout, 2, 2>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc);
-    case 8: return stream ? inv4s<Tc, TU, Tout, 4, 2>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc)
-                    : inv4<Tc, TU, Tout, 4, 2>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc);
-    case 16: return stream ? inv4s<Tc, TU, Tout, 4, 4>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc)
-                    : inv4<Tc, TU, Tout, 4, 4>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc);
-    case 32: return stream ? inv4s<Tc, TU, Tout, 8, 4>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc)
-                    : inv4<Tc, TU, Tout, 8, 4>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc);
-    case 64: return stream ? inv4s<Tc, TU, Tout, 8, 8>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc)
-                    : inv4<Tc, TU, Tout, 8, 8>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc);
-    case 128: return stream ? inv4s<Tc, TU, Tout, 16, 8>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc)
-                    : inv4<Tc, TU, Tout, 16, 8>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc);
-    case 256: return stream ? inv4s<Tc, TU, Tout, 16, 16>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc)
-                    : inv4<Tc, TU, Tout, 16, 16>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc);
+    case 1: return stream ? inv4s<Tc, TU, Tout, 1, 1>(L, ms, spec, dinv, tw, w, wstride, jdev, fc)
+                    : inv4<Tc, TU, Tout, 1, 1>(L, ms, spec, dinv, tw, w, wstride, jdev, fc);
+    case 2: return stream ? inv4s<Tc, TU, Tout, 2, 1>(L, ms, spec, dinv, tw, w, wstride, jdev, fc)
+                    : inv4<Tc, TU, Tout, 2, 1>(L, ms, spec, dinv, tw, w, wstride, jdev, fc);
+    case 4: return stream ? inv4s<Tc, TU, Tout, 2, 2>(L, ms, spec, dinv, tw, w, wstride, jdev, fc)
+                    : inv4<Tc, TU, Tout, 2, 2>(L, ms, spec, dinv, tw, w, wstride, jdev, fc);
+    case 8: return stream ? inv4s<Tc, TU, Tout, 4, 2>(L, ms, spec, dinv, tw, w, wstride, jdev, fc)
+                    : inv4<Tc, TU, Tout, 4, 2>(L, ms, spec, dinv, tw, w, wstride, jdev, fc);
+    case 16: return stream ? inv4s<Tc, TU, Tout, 4, 4>(L, ms, spec, dinv, tw, w, wstride, jdev, fc)
+                    : inv4<Tc, TU, Tout, 4, 4>(L, ms, spec, dinv, tw, w, wstride, jdev, fc);
+    case 32: return stream ? inv4s<Tc, TU, Tout, 8, 4>(L, ms, spec, dinv, tw, w, wstride, jdev, fc)
+                    : inv4<Tc, TU, Tout, 8, 4>(L, ms, spec, dinv, tw, w, wstride, jdev, fc);
+    case 64: return stream ? inv4s<Tc, TU, Tout, 8, 8>(L, ms, spec, dinv, tw, w, wstride, jdev, fc)
+                    : inv4<Tc, TU, Tout, 8, 8>(L, ms, spec, dinv, tw, w, wstride, jdev, fc);
+    case 128: return stream ? inv4s<Tc, TU, Tout, 16, 8>(L, ms, spec, dinv, tw, w, wstride, jdev, fc)
+                    : inv4<Tc, TU, Tout, 16, 8>(L, ms, spec, dinv, tw, w, wstride, jdev, fc);
+    case 256: return stream ? inv4s<Tc, TU, Tout, 16, 16>(L, ms, spec, dinv, tw, w, wstride, jdev, fc)
+                    : inv4<Tc, TU, Tout, 16, 16>(L, ms, spec, dinv, tw, w, wstride, jdev, fc);
     case 512:
-      if constexpr (sizeof(Tc) == 4) return stream ? inv4s<Tc, TU, Tout, 32, 16>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc)
-                    : inv4<Tc, TU, Tout, 32, 16>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc);
+      if constexpr (sizeof(Tc) == 4) return stream ? inv4s<Tc, TU, Tout, 32, 16>(L, ms, spec, dinv, tw, w, wstride, jdev, fc)
+                    : inv4<Tc, TU, Tout, 32, 16>(L, ms, spec, dinv, tw, w, wstride, jdev, fc);
       break;
     case 1024:
-      if constexpr (sizeof(Tc) == 4) return stream ? inv4s<Tc, TU, Tout, 32, 32>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc)
-                    : inv4<Tc, TU, Tout, 32, 32>(L, ms, spec, dpow, dinv, tw, w, wstride, jdev, fc);
+      if constexpr (sizeof(Tc) == 4) return stream ? inv4s<Tc, TU, Tout, 32, 32>(L, ms, spec, dinv, tw, w, wstride, jdev, fc)
+                    : inv4<Tc, TU, Tout, 32, 32>(L, ms, spec, dinv, tw, w, wstride, jdev, fc);
       break;
   }
   return cudaErrorInvalidValue;
 }
 
 template <typename Tc, typename Tin>
-cudaError_t launch_tfft_forward(Launch& L, int64_t ms, int n, const Tin* v, const Tc* dpow, const Tc* dinv,
+cudaError_t launch_tfft_forward(Launch& L, int64_t ms, int n, const Tin* v, const Tc* dpow,
                                 const typename Cx<Tc>::t* tw, typename Cx<Tc>::t* spec, size_t vstride,
                                 const int* jdev) {
   const bool pow2 = (n & (n - 1)) == 0;
@@ -826,7 +819,7 @@ cudaError_t launch_tfft_forward(Launch& L, int64_t ms, int n, const Tin* v, cons
     if (e != cudaSuccess) return e;
     const int nf = n / 2 + 1;
     L.begin(KC_TFFT_FWD);
-    tdft_forward_kernel<Tc, Tin><<<(unsigned)((ms + TS - 1) / TS), 256, smem, L.stream>>>(v, dpow, dinv, tw, spec, ms, n, TS);
+    tdft_forward_kernel<Tc, Tin><<<(unsigned)((ms + TS - 1) / TS), 256, smem, L.stream>>>(v, dpow, tw, spec, ms, n, TS);
     return L.end(KC_TFFT_FWD, 2.0 * n * ms * sizeof(Tin) + 2.0 * nf * ms * sizeof(typename Cx<Tc>::t),
                  16.0 * (double)nf * n * ms);
   }
@@ -835,7 +828,7 @@ cudaError_t launch_tfft_forward(Launch& L, int64_t ms, int n, const Tin* v, cons
     const double bytes = 2.0 * n * ms * sizeof(Tin) + 2.0 * nf * ms * sizeof(typename Cx<Tc>::t);
     const double flops = (double)ms * (5.0 * n * ilog2(n) + 2.0 * n);
     L.begin(KC_TFFT_FWD);
-    fwd4_dispatch<Tin, Tc>(L, ms, n, v, dpow, dinv, tw, spec, vstride, jdev);
+    fwd4_dispatch<Tin, Tc>(L, ms, n, v, dpow, tw, spec, vstride, jdev);
     return L.end(KC_TFFT_FWD, bytes, flops);
   }
   const int TS = pick_ts<Tc>(n);
@@ -867,7 +860,7 @@ cudaError_t launch_tfft_inverse(Launch& L, int64_t ms, int n, const TU* spec, co
     if (e != cudaSuccess) return e;
     const int nf = n / 2 + 1;
     L.begin(KC_TFFT_INV);
-    tdft_inverse_kernel<Tc, TU, Tout><<<(unsigned)((ms + TS - 1) / TS), 256, smem, L.stream>>>(spec, dpow, dinv, tw, w,
+    tdft_inverse_kernel<Tc, TU, Tout><<<(unsigned)((ms + TS - 1) / TS), 256, smem, L.stream>>>(spec, dinv, tw, w,
                                                                                             ms, n, TS, fc);
     return L.end(KC_TFFT_INV, 2.0 * nf * ms * sizeof(TU) + 2.0 * n * ms * sizeof(Tout) + cbytes,
                  8.0 * (double)n * n * ms);
@@ -877,7 +870,7 @@ cudaError_t launch_tfft_inverse(Launch& L, int64_t ms, int n, const TU* spec, co
     const double bytes = 2.0 * nf * ms * sizeof(TU) + 2.0 * n * ms * sizeof(Tout) + cbytes;
     const double flops = (double)ms * (5.0 * n * ilog2(n) + 4.0 * n);
     L.begin(KC_TFFT_INV);
-    inv4_dispatch<Tc, TU, Tout>(L, ms, n, spec, dpow, dinv, tw, w, wstride, jdev, fc);
+    inv4_dispatch<Tc, TU, Tout>(L, ms, n, spec, dinv, tw, w, wstride, jdev, fc);
     return L.end(KC_TFFT_INV, bytes, flops);
   }
   const int TS = pick_ts<Tc>(n);
@@ -894,11 +887,11 @@ cudaError_t launch_tfft_inverse(Launch& L, int64_t ms, int n, const TU* spec, co
 }
 
 template cudaError_t launch_tfft_forward<double, double>(Launch&, int64_t, int, const double*, const double*,
-                                                         const double*, const double2*, double2*, size_t, const int*);
+                                                         const double2*, double2*, size_t, const int*);
 template cudaError_t launch_tfft_forward<float, double>(Launch&, int64_t, int, const double*, const float*,
-                                                        const float*, const float2*, float2*, size_t, const int*);
+                                                        const float2*, float2*, size_t, const int*);
 template cudaError_t launch_tfft_forward<float, float>(Launch&, int64_t, int, const float*, const float*,
-                                                       const float*, const float2*, float2*, size_t, const int*);
+                                                       const float2*, float2*, size_t, const int*);
 #define PCOPT_INV(Tc, TU, Tout)                                                                                  \
   template cudaError_t launch_tfft_inverse<Tc, TU, Tout>(Launch&, int64_t, int, const TU*, const Tc*, const Tc*, \
                                                          const Cx<Tc>::t*, Tout*, size_t, const int*,         \
