@@ -1662,8 +1662,9 @@ static int gmres_impl(pc_handle* h, const double* b, double* x, double rtol, int
   // Iteration j = front (z_j = P^{-1} v_j and w = A z_j, or the left-preconditioned
   // pair; it needs only v_j) + back (Arnoldi passes, Givens, the estimate copied to
   // mapped host memory behind an event, which the host waits for).  Queuing the next
-  // front before that wait was tried: the GPU never idled long enough for it to pay
-  // (0.0852 vs 0.0849 s per solve at 255^2 x 256), so the next front waits for the decision.
+  // front before that wait was tried at 255^2 x 256 alone, where the GPU does not idle long
+  // enough for it to pay (0.0852 vs 0.0849 s per solve): the next front waits for the
+  // decision.  At 31^2 x 32, where the GPU does idle, it has not been measured.
   auto front = [&](int j) -> cudaError_t {
     double* vj = V + (size_t)j * U;
     double* vn = V + (size_t)(j + 1) * U;

@@ -9,6 +9,8 @@
 // 2 x 344 + 35 -> 452.  FP32, bound elsewhere, takes all m products of an output, j ascending:
 // a solve preconditioned in FP32 stops where FP32 rounding, amplified by A, stands at rtol, so
 // with sums and differences its solution moves by up to rtol (30^2 x 50 at rtol = 1e-8: 1e-8).
+// 100^2 x 102 planes in FP32: an axis pass 102 us with one thread a value, 43 from tiles (39
+// with half the products), the fused last axis 69 (73).
 //
 // A CTA of 256 threads holds a tile of lines in shared memory, the line index fastest; a
 // thread forms up to four outputs (FP64: of one parity) of its line at a time.  S is read

@@ -88,9 +88,8 @@ __global__ void __launch_bounds__(256) matvec_kernel(const Tin* __restrict__ x, 
     const double k1 = tauK(x1 + idx, x1c);
     const double k2 = tauK(x2 + idx, x2c);
     // The difference in time is formed first: it is exact for vectors smooth in time, and 1 + d
-    // as one coefficient (an operation less: 255^2 x 256 at 32 blocks a thread 431 us instead of
-    // 498) rounds at the size of v before the difference cancels, up to 60 times this error
-    // where d is small.
+    // as one coefficient (an operation less: 255^2 x 256 420 us instead of 474) rounds at the
+    // size of v before the difference cancels, up to 60 times this error where d is small.
     const double tT_x2 = x2c - x2n + k2;     // (T^T x2)_j
     const double t_x1 = x1c - x1prev + k1;   // (T x1)_j
     y1[idx] = fma(alpha, x1c, TRANSPOSE ? -tT_x2 : tT_x2);
@@ -105,8 +104,8 @@ __global__ void __launch_bounds__(256) matvec_kernel(const Tin* __restrict__ x, 
 // Time blocks per thread: the tuned value, else 4 for the FP64 kernel.  A thread re-reads
 // two x values and its stencil at the start of a chunk; the FP64 unit bounds the kernel,
 // so that costs little at any size, and short chunks fill the chip where n is small
-// (63^2 x 64: 34.8 us at 32 blocks a thread, 12.3 at 4; 127^2 x 128: 63.6 and 57.4;
-// 255^2 x 256: 431 and 419; one block a thread takes 445 there).
+// (63^2 x 64: 39.0 us at 32 blocks a thread, 12.4 at 4 and at 1; 127^2 x 128: 73.8, 65.5 and
+// 63.5; 255^2 x 256: 497, 474 and 472).
 static int time_chunk(const Launch& L, int n) {
   const int tj = L.tiles && L.tiles->mv_tj > 0 ? L.tiles->mv_tj : 4;
   return tj < n ? tj : n;
