@@ -129,7 +129,7 @@ typedef struct pc_params {
   int m1;           /* interior grid points per dimension, h = 1/(m1+1); multigrid needs m1 = 2^k-1 */
   int n;            /* time blocks (FFT length), tau = T/(n+1); 1..4096.  Powers of two use the
                        register FFT; other lengths (the paper's n = 2^k - 1) the chirp-z method
-                       (n < 24: a direct DFT) */
+                       (n < 24, and FP32 around sine-transform solves or BF16 storage: a direct DFT) */
   double T;         /* final time > 0 */
   double gamma;     /* regularisation parameter > 0 */
   double eps;       /* eps of C_{eps,n}, in (0, 1] */
